@@ -542,14 +542,23 @@ static size_t bwg_smem() {
 // K < kKPad leaves basis column K zero
 bool edge_tc_supported(int F, int K) { return F == kF && K < kKPad && K >= 2; }
 
-// Rows per block-cyclic chunk: the context's setting, or one contiguous range per stream (0).
-static int64_t chunk_rows_for(const ModelW& m, int64_t n, int ns) {
-  if (m.edge_chunk_rows > 0) return m.edge_chunk_rows;
+static int sm_count() {
   int dev = 0, sms = 148;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  const int64_t streams = (int64_t)sms * ns;
-  const int64_t r = (n + streams - 1) / streams;
+  return sms;
+}
+
+// Rows per block-cyclic chunk.  The context's setting (0: one contiguous range per stream) is the
+// largest chunk; with w = ceil(n / (streams * setting)) chunks per stream, n is cut evenly into
+// streams * w chunks, so that every stream gets rows when there are few (500 atoms on 304 streams:
+// 2 rows each instead of 32 rows on 16 of them, 18 us per launch instead of 174) and none gets a chunk more than it
+// must when there are some thousands.  At 1M atoms the chunk stays at 32 rows.
+static int64_t chunk_rows_for(const ModelW& m, int64_t n, int ns) {
+  const int64_t streams = (int64_t)sm_count() * ns;
+  const int64_t most = m.edge_chunk_rows > 0 ? m.edge_chunk_rows : n;
+  const int64_t w = (n + streams * most - 1) / (streams * most);
+  const int64_t r = (n + streams * w - 1) / (streams * w);
   return r > 0 ? r : 1;
 }
 
@@ -572,9 +581,7 @@ int edge_bwd_tc(cudaStream_t st, const ModelW& m, int t, int accumulate, int64_t
     cudaFuncSetAttribute(k_edge_bwd_tcg<kBwgNE, kBwgNS, 20, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bwg_smem());
     attr = true;
   }
-  int sms = 0, dev = 0;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  const int sms = sm_count();
   const int threads = 32 * (3 + 4 * kBwgNS);
   LaunchScope ls_(st);
   if (m.K == 20 && t == 0 && !GPHI)   // the usual basis size; first layer: v = 0, no phi gradients
