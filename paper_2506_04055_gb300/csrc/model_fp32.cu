@@ -36,6 +36,24 @@ namespace ctd {
 enum Epi { EPI_BIAS = 0, EPI_BIAS_SILU = 1, EPI_ADD = 2, EPI_DSILU = 3 };
 constexpr int GBM = 64, GBN = 128, GBK = 32;
 
+// Four outputs of row m, columns nb .. nb + 3, with the fused epilogue.
+template <int EPI>
+__device__ __forceinline__ void gemm_store(const float (&acc)[4], int64_t m, int nb, const float* bias, const float* aux,
+                                           int ldaux, float* out, int ldo, float* out2, int ldo2) {
+  float r[4];
+#pragma unroll
+  for (int j = 0; j < 4; ++j) {
+    float x = acc[j];
+    if (EPI == EPI_BIAS || EPI == EPI_BIAS_SILU) x += bias ? bias[nb + j] : 0.0f;
+    if (EPI == EPI_ADD) x += aux[m * ldaux + nb + j];
+    if (EPI == EPI_DSILU) x *= dsilu_f(aux[m * ldaux + nb + j]);
+    r[j] = x;
+  }
+  *reinterpret_cast<float4*>(&out[m * ldo + nb]) = make_float4(r[0], r[1], r[2], r[3]);
+  if (EPI == EPI_BIAS_SILU)
+    *reinterpret_cast<float4*>(&out2[m * ldo2 + nb]) = make_float4(silu_f(r[0]), silu_f(r[1]), silu_f(r[2]), silu_f(r[3]));
+}
+
 template <int EPI, int BN = GBN>
 __global__ __launch_bounds__(256) void k_gemm(int64_t M, int N, int K, const float* __restrict__ A, int lda,
                                               const float* __restrict__ B, const float* __restrict__ bias,
@@ -102,77 +120,155 @@ __global__ __launch_bounds__(256) void k_gemm(int64_t M, int N, int K, const flo
   for (int i = 0; i < 8; ++i) {
     int64_t m = m0 + ty * 8 + i;
     if (m >= M) break;
-    float r[4];
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      float x = acc[i][j];
-      if (EPI == EPI_BIAS || EPI == EPI_BIAS_SILU) x += bias ? bias[nb + j] : 0.0f;
-      if (EPI == EPI_ADD) x += aux[m * ldaux + nb + j];
-      if (EPI == EPI_DSILU) x *= dsilu_f(aux[m * ldaux + nb + j]);
-      r[j] = x;
-    }
-    *reinterpret_cast<float4*>(&out[m * ldo + nb]) = make_float4(r[0], r[1], r[2], r[3]);
-    if (EPI == EPI_BIAS_SILU)
-      *reinterpret_cast<float4*>(&out2[m * ldo2 + nb]) =
-          make_float4(silu_f(r[0]), silu_f(r[1]), silu_f(r[2]), silu_f(r[3]));
+    gemm_store<EPI>(acc[i], m, nb, bias, aux, ldaux, out, ldo, out2, ldo2);
   }
 }
 
-// Small problems (fewer output tiles than one wave of the GPU): one thread per output element,
-// the same fmaf chain over k in increasing order and the same epilogue as k_gemm, so results
-// are bit for bit those of the tiled kernel, with more warps in flight than its few CTAs.
-template <int EPI>
-__global__ void k_gemm_small(int64_t M, int N, int K, const float* __restrict__ A, int lda,
-                             const float* __restrict__ B, const float* __restrict__ bias,
-                             const float* __restrict__ aux, int ldaux, float* __restrict__ out, int ldo,
-                             float* __restrict__ out2, int ldo2) {
-  const int64_t idx = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (idx >= M * N) return;
-  const int64_t m = idx / N;
-  const int n = (int)(idx % N);
-  const float* a = A + m * lda;
-  float x = 0.0f;
-  for (int k = 0; k < K; ++k) x = fmaf(__ldg(a + k), __ldg(B + (int64_t)k * N + n), x);
-  if (EPI == EPI_BIAS || EPI == EPI_BIAS_SILU) x += bias ? bias[n] : 0.0f;
-  if (EPI == EPI_ADD) x += aux[m * ldaux + n];
-  if (EPI == EPI_DSILU) x *= dsilu_f(aux[m * ldaux + n]);
-  out[m * ldo + n] = x;
-  if (EPI == EPI_BIAS_SILU) out2[m * ldo2 + n] = silu_f(x);
+__device__ __forceinline__ void cp_async16_zfill(void* dst, const void* src, bool live) {
+  const uint32_t d = static_cast<uint32_t>(__cvta_generic_to_shared(dst));
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(d), "l"(src), "r"(live ? 16 : 0) : "memory");
+}
+template <int N>
+__device__ __forceinline__ void cp_async_wait() {
+  asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
 }
 
-template <int EPI, int BN = GBN>
-static void gemm(cudaStream_t st, int64_t M, int N, int K, const float* A, int lda, const float* B,
-                 const float* bias, const float* aux, int ldaux, float* out, int ldo, float* out2 = nullptr,
-                 int ldo2 = 0) {
+// Small problems: BM x BN output tiles, TM rows x 4 columns per thread.  They are bound by latency
+// (one wave or less of tiles, K = 64 .. 768), so the whole K extent of both operands is put in
+// flight at once with cp.async, in 64-deep commit groups, and the chain over k starts as soon as
+// the first group has landed: one memory latency per launch.  The thread-per-output kernel that
+// stood here walked K with a global load per step (192 atoms, F = 64: 13 to 33 us per launch, now
+// 4.4 to 7.3; 5,997 atoms: 23 to 47 us, now 8 to 15).
+// Same fmaf chain over k in increasing order and same epilogue as k_gemm: bit-identical outputs.
+constexpr int GSK = 64;   // k per commit group
+template <int BM, int BN>
+static size_t gemm_small_smem(int K) {
+  return sizeof(float) * ((size_t)BM * (K + 4) + (size_t)K * BN);
+}
+template <int EPI, int BM, int BN, int TM>
+__global__ __launch_bounds__((BM / TM) * (BN / 4)) void k_gemm_small(
+    int64_t M, int N, int K, const float* __restrict__ A, int lda, const float* __restrict__ B,
+    const float* __restrict__ bias, const float* aux, int ldaux, float* out, int ldo, float* __restrict__ out2, int ldo2) {
+  constexpr int NT = (BM / TM) * (BN / 4), TX = BN / 4;
+  extern __shared__ float4 gs_smem4[];
+  float* As = reinterpret_cast<float*>(gs_smem4);   // [BM][K + 4]
+  const int ldk = K + 4;
+  float* Bs = As + (size_t)BM * ldk;                // [K][BN]
+  const int tid = threadIdx.x, tx = tid % TX, ty = tid / TX;
+  const int ncol = (N + BN - 1) / BN;
+  const int64_t m0 = (int64_t)(blockIdx.x / ncol) * BM;
+  const int n0 = (int)(blockIdx.x % ncol) * BN;
+  const int ngroups = (K + GSK - 1) / GSK;
+  for (int c = 0; c < ngroups; ++c) {
+    const int k0 = c * GSK, kc = K - k0 < GSK ? K - k0 : GSK, kc4 = kc >> 2;   // K is a multiple of 4
+    for (int idx = tid; idx < BM * kc4; idx += NT) {
+      const int r = idx / kc4, q = k0 + 4 * (idx % kc4);
+      const bool live = m0 + r < M;
+      cp_async16_zfill(As + r * ldk + q, A + (live ? (m0 + r) * lda + q : 0), live);
+    }
+    for (int idx = tid; idx < kc * TX; idx += NT) {
+      const int r = k0 + idx / TX, q = 4 * (idx % TX);
+      const bool live = n0 + q < N;
+      cp_async16_zfill(Bs + r * BN + q, B + (live ? (int64_t)r * N + n0 + q : 0), live);
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  }
+  float acc[TM][4];
+#pragma unroll
+  for (int i = 0; i < TM; ++i)
+#pragma unroll
+    for (int j = 0; j < 4; ++j) acc[i][j] = 0.0f;
+  for (int c = 0; c < ngroups; ++c) {
+    // groups complete in order; the last four are told apart, earlier ones wait for more than needed
+    switch (ngroups - 1 - c) {
+      case 0: cp_async_wait<0>(); break;
+      case 1: cp_async_wait<1>(); break;
+      case 2: cp_async_wait<2>(); break;
+      default: cp_async_wait<3>(); break;
+    }
+    __syncthreads();
+    const int k1 = K < (c + 1) * GSK ? K : (c + 1) * GSK;
+#pragma unroll 4
+    for (int k = c * GSK; k < k1; k += 4) {
+      float av[TM][4];
+#pragma unroll
+      for (int i = 0; i < TM; ++i) {
+        const float4 a = *reinterpret_cast<const float4*>(As + (ty * TM + i) * ldk + k);
+        av[i][0] = a.x; av[i][1] = a.y; av[i][2] = a.z; av[i][3] = a.w;
+      }
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const float4 b = *reinterpret_cast<const float4*>(Bs + (k + q) * BN + tx * 4);
+#pragma unroll
+        for (int i = 0; i < TM; ++i) {
+          acc[i][0] = fmaf(av[i][q], b.x, acc[i][0]);
+          acc[i][1] = fmaf(av[i][q], b.y, acc[i][1]);
+          acc[i][2] = fmaf(av[i][q], b.z, acc[i][2]);
+          acc[i][3] = fmaf(av[i][q], b.w, acc[i][3]);
+        }
+      }
+    }
+  }
+  const int nb = n0 + tx * 4;
+  if (nb >= N) return;
+#pragma unroll
+  for (int i = 0; i < TM; ++i) {
+    const int64_t m = m0 + ty * TM + i;
+    if (m < M) gemm_store<EPI>(acc[i], m, nb, bias, aux, ldaux, out, ldo, out2, ldo2);
+  }
+}
+
+constexpr int kMidK = 512, kSmallK = 768;   // largest K of the two tile shapes (3F = 768 at F = 256)
+template <int EPI, int BM, int BN, int TM>
+static void launch_gemm_small(cudaStream_t st, int64_t M, int N, int K, const float* A, int lda, const float* B,
+                              const float* bias, const float* aux, int ldaux, float* out, int ldo, float* out2, int ldo2) {
+  static const cudaError_t attr = cudaFuncSetAttribute(
+      k_gemm_small<EPI, BM, BN, TM>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+      (int)gemm_small_smem<BM, BN>(BM == 32 ? kMidK : kSmallK));
+  (void)attr;
+  const unsigned grid = (unsigned)(((M + BM - 1) / BM) * ((N + BN - 1) / BN));
+  LaunchScope ls_(st);
+  k_gemm_small<EPI, BM, BN, TM><<<grid, (BM / TM) * (BN / 4), gemm_small_smem<BM, BN>(K), st>>>(
+      M, N, K, A, lda, B, bias, aux, ldaux, out, ldo, out2, ldo2);
+}
+
+template <int EPI, int BN>
+static void gemm_tiled(cudaStream_t st, int64_t M, int N, int K, const float* A, int lda, const float* B,
+                       const float* bias, const float* aux, int ldaux, float* out, int ldo, float* out2, int ldo2) {
   if (M == 0) return;
   constexpr int BM = 8 * (256 / (BN / 4));
   const int64_t tiles = (int64_t)((N + BN - 1) / BN) * ((M + BM - 1) / BM);
-  if (tiles < 152) {
-    LaunchScope ls_(st);
-    k_gemm_small<EPI><<<(unsigned)((M * N + 255) / 256), 256, 0, st>>>(M, N, K, A, lda, B, bias, aux, ldaux, out,
-                                                                     ldo, out2, ldo2);
+  if (tiles < 2 * 152 && K <= kSmallK) {   // under two waves of the 256-thread tiles
+    const int64_t mid = ((M + 31) / 32) * ((N + 63) / 64);
+    // 32 x 64 tiles once they fill the SMs, 16 x 32 tiles below that
+    if (mid >= 152 && K <= kMidK)
+      launch_gemm_small<EPI, 32, 64, 4>(st, M, N, K, A, lda, B, bias, aux, ldaux, out, ldo, out2, ldo2);
+    else
+      launch_gemm_small<EPI, 16, 32, 1>(st, M, N, K, A, lda, B, bias, aux, ldaux, out, ldo, out2, ldo2);
     return;
   }
-  { LaunchScope ls_(st); k_gemm<EPI, BN><<<(unsigned)tiles, 256, 0, st>>>(M, N, K, A, lda, B, bias, aux, ldaux, out, ldo, out2, ldo2); }
+  LaunchScope ls_(st);
+  k_gemm<EPI, BN><<<(unsigned)tiles, 256, 0, st>>>(M, N, K, A, lda, B, bias, aux, ldaux, out, ldo, out2, ldo2);
 }
 
 // The tile width follows N (32, 64 or 128 columns), so narrow outputs do not compute idle
 // columns; the results are those of the 128-column tile, bit for bit.
-template <int BN>
-static void gemm_epi(cudaStream_t st, int epi, int64_t M, int N, int K, const float* A, int lda, const float* B,
-                     const float* bias, const float* aux, int ldaux, float* out, int ldo, float* out2, int ldo2) {
-  switch (epi) {
-    case EPI_BIAS: gemm<EPI_BIAS, BN>(st, M, N, K, A, lda, B, bias, aux, ldaux, out, ldo, out2, ldo2); break;
-    case EPI_BIAS_SILU: gemm<EPI_BIAS_SILU, BN>(st, M, N, K, A, lda, B, bias, aux, ldaux, out, ldo, out2, ldo2); break;
-    case EPI_ADD: gemm<EPI_ADD, BN>(st, M, N, K, A, lda, B, bias, aux, ldaux, out, ldo, out2, ldo2); break;
-    default: gemm<EPI_DSILU, BN>(st, M, N, K, A, lda, B, bias, aux, ldaux, out, ldo, out2, ldo2); break;
-  }
+template <int EPI>
+static void gemm(cudaStream_t st, int64_t M, int N, int K, const float* A, int lda, const float* B,
+                 const float* bias, const float* aux, int ldaux, float* out, int ldo, float* out2 = nullptr,
+                 int ldo2 = 0) {
+  if (N <= 32) gemm_tiled<EPI, 32>(st, M, N, K, A, lda, B, bias, aux, ldaux, out, ldo, out2, ldo2);
+  else if (N <= 64) gemm_tiled<EPI, 64>(st, M, N, K, A, lda, B, bias, aux, ldaux, out, ldo, out2, ldo2);
+  else gemm_tiled<EPI, 128>(st, M, N, K, A, lda, B, bias, aux, ldaux, out, ldo, out2, ldo2);
 }
 void gemm_f32(cudaStream_t st, int epi, int64_t M, int N, int K, const float* A, int lda, const float* B,
               const float* bias, const float* aux, int ldaux, float* out, int ldo, float* out2, int ldo2) {
-  if (N <= 32) gemm_epi<32>(st, epi, M, N, K, A, lda, B, bias, aux, ldaux, out, ldo, out2, ldo2);
-  else if (N <= 64) gemm_epi<64>(st, epi, M, N, K, A, lda, B, bias, aux, ldaux, out, ldo, out2, ldo2);
-  else gemm_epi<128>(st, epi, M, N, K, A, lda, B, bias, aux, ldaux, out, ldo, out2, ldo2);
+  switch (epi) {
+    case EPI_BIAS: gemm<EPI_BIAS>(st, M, N, K, A, lda, B, bias, aux, ldaux, out, ldo, out2, ldo2); break;
+    case EPI_BIAS_SILU: gemm<EPI_BIAS_SILU>(st, M, N, K, A, lda, B, bias, aux, ldaux, out, ldo, out2, ldo2); break;
+    case EPI_ADD: gemm<EPI_ADD>(st, M, N, K, A, lda, B, bias, aux, ldaux, out, ldo, out2, ldo2); break;
+    default: gemm<EPI_DSILU>(st, M, N, K, A, lda, B, bias, aux, ldaux, out, ldo, out2, ldo2); break;
+  }
 }
 
 // ================================================================================ node kernels
