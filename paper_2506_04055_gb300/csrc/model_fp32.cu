@@ -916,159 +916,172 @@ static bool readout_is_fused(int F) { return F == 64 || F == 128; }
 // E_i = e_scale w_i (R2 . silu(h) + d2) and, with gradients, g = w_i e_scale R2 * silu'(h) and
 // gs = R1^T g, h and gs as FP32 fmaf chains over the inputs and over the hidden units in order
 // (as the GEMMs they replace), the energy terms in FP64, summed over the 16 threads that hold an
-// atom's units in a fixed tree (so independent of the launch).  A block of 512 threads stands for one
-// 256-thread block of the grid-stride energy sum: it takes the 256-atom ranges starting at
-// 256 (b + G k) (G = blocks), as two 128-atom tiles, and its thread t < 256 adds the energy of
-// atom 256 (b + G k) + t, the same atoms in the same order.  s and R1 are staged transposed so
-// that each thread's 4 atoms and 4 units come in 16-byte shared loads.
-template <int F>
-__global__ __launch_bounds__(512, 1) void k_readout_fused(int64_t n, float e_scale, const float* __restrict__ S,
+// atom's units in a fixed tree (so independent of the launch).  A block of 4 TA threads takes the
+// TA-atom tiles starting at TA (b + G k) (G = blocks), thread t < TA adding the energy of atom
+// TA (b + G k) + t; blocks beyond the last tile only write a zero partial.  s and R1 are staged
+// transposed so that each thread's 4 atoms and 4 units come in 16-byte shared loads.  TA = 128 keeps
+// the weights' shared loads per atom low; below one such tile per SM, TA = 32 spreads the atoms over
+// four times the SMs (192 atoms, F = 64: 13 us against 30; 500 atoms, F = 128: 25 against 63).
+template <int F, int TA>
+__global__ __launch_bounds__(4 * TA, 1) void k_readout_fused(int64_t n, float e_scale, const float* __restrict__ S,
                                                        const float* __restrict__ R1, const float* __restrict__ R1t,
                                                        const float* __restrict__ d1, const float* __restrict__ R2,
                                                        const float* __restrict__ d2, const float* __restrict__ ew,
                                                        float* __restrict__ GS, float* __restrict__ e_atom,
                                                        double* __restrict__ partials) {
-  constexpr int FH = F / 2, TA = 128, F4 = F / 4, GP = FH + 4;
+  constexpr int FH = F / 2, F4 = F / 4, GP = FH + 4, NT = 4 * TA;
   constexpr int OPT = FH / 16, KPT = F / 16;   // units (forward) and inputs (backward) per thread
   extern __shared__ float4 rd_smem4[];
   float* sR1T = reinterpret_cast<float*>(rd_smem4);   // [F][FH]   R1^T (input, unit)
   float* sR1 = sR1T + F * FH;                         // [FH][F]   R1 (unit, input)
   float* sST = sR1 + FH * F;                          // [F][TA]   s^T of the tile
   float* sG = sST + F * TA;                           // [TA][GP]  g of the tile
-  float* sE = sG + TA * GP;                           // [256]     per-atom energies of the range
-  float* sR2 = sE + 256;                              // [FH]
-  __shared__ double sbuf[8];
+  float* sE = sG + TA * GP;                           // [TA]      per-atom energies of the tile
+  float* sR2 = sE + TA;                               // [FH]
+  __shared__ double sbuf[TA / 32];
   const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;   // ty: atoms 4 ty .. 4 ty + 3
-  for (int idx = tid; idx < F * FH / 4; idx += 512) {
+  if ((int64_t)blockIdx.x * TA >= n) {   // uniform over the block
+    if (tid == 0) partials[blockIdx.x] = 0.0;
+    return;
+  }
+  for (int idx = tid; idx < F * FH / 4; idx += NT) {
     reinterpret_cast<float4*>(sR1T)[idx] = reinterpret_cast<const float4*>(R1t)[idx];
     reinterpret_cast<float4*>(sR1)[idx] = reinterpret_cast<const float4*>(R1)[idx];
   }
-  for (int k = tid; k < FH; k += 512) sR2[k] = R2[k];
+  for (int k = tid; k < FH; k += NT) sR2[k] = R2[k];
   __syncthreads();
   double acc = 0.0, comp = 0.0;
-  const int64_t G = (int64_t)gridDim.x * 256;
-  for (int64_t base = (int64_t)blockIdx.x * 256; base < n; base += G) {
-    for (int t2 = 0; t2 < 2; ++t2) {
-      const int64_t a0 = base + t2 * TA;
-      for (int idx = tid; idx < TA * F4; idx += 512) {
-        const int a = idx % TA, k4 = idx / TA;
-        float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (a0 + a < n) v = reinterpret_cast<const float4*>(S + (a0 + a) * F)[k4];
-        sST[(4 * k4 + 0) * TA + a] = v.x;
-        sST[(4 * k4 + 1) * TA + a] = v.y;
-        sST[(4 * k4 + 2) * TA + a] = v.z;
-        sST[(4 * k4 + 3) * TA + a] = v.w;
-      }
-      __syncthreads();
-      {
-        float h[4][OPT];
-#pragma unroll
-        for (int i = 0; i < 4; ++i)
-#pragma unroll
-          for (int j = 0; j < OPT; ++j) h[i][j] = 0.0f;
-#pragma unroll 4
-        for (int k = 0; k < F; ++k) {
-          const float4 sa = *reinterpret_cast<const float4*>(sST + k * TA + 4 * ty);
-          float r[OPT];
-          if constexpr (OPT == 4) {
-            const float4 q = *reinterpret_cast<const float4*>(sR1T + k * FH + 4 * tx);
-            r[0] = q.x; r[1] = q.y; r[2] = q.z; r[3] = q.w;
-          } else {
-            const float2 q = *reinterpret_cast<const float2*>(sR1T + k * FH + 2 * tx);
-            r[0] = q.x; r[1] = q.y;
-          }
-          const float sv[4] = {sa.x, sa.y, sa.z, sa.w};
-#pragma unroll
-          for (int i = 0; i < 4; ++i)
-#pragma unroll
-            for (int j = 0; j < OPT; ++j) h[i][j] = fmaf(sv[i], r[j], h[i][j]);
-        }
-        // energy terms of this thread's units, each product split exactly (FMA) and added into a
-        // float-float pair (TwoSum), the pairs of the 16 threads of an atom combined in a fixed
-        // tree: the terms can largely cancel, and this keeps ~44 bits of their sum without the
-        // FP64 pipe; g = w e_scale R2 silu'(h) goes to the g tile
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-          const int64_t ai = a0 + 4 * ty + i;
-          const float wi = ai < n && ew ? ew[ai] : 1.0f;
-          float es = 0.0f, ec = 0.0f;
-#pragma unroll
-          for (int j = 0; j < OPT; ++j) {
-            const int o = OPT * tx + j;
-            const float hk = h[i][j] + (d1 ? d1[o] : 0.0f);
-            const float sl = silu_f(hk), pr = __fmul_rn(sR2[o], sl);
-            ff_add(es, ec, pr, __fmaf_rn(sR2[o], sl, -pr));
-            if (GS) sG[(4 * ty + i) * GP + o] = ai < n ? wi * (e_scale * sR2[o] * dsilu_f(hk)) : 0.0f;
-          }
-#pragma unroll
-          for (int off = 1; off < 16; off <<= 1) {
-            const float os = __shfl_xor_sync(0xffffffffu, es, off), oc = __shfl_xor_sync(0xffffffffu, ec, off);
-            ff_add(es, ec, os, oc);
-          }
-          if (tx == 0) {
-            double e = ((double)es + (double)ec + (double)d2[0]) * (double)e_scale;
-            e *= (double)wi;
-            const float ef = ai < n ? (float)e : 0.0f;
-            if (ai < n && e_atom) e_atom[ai] = ef;
-            sE[t2 * TA + 4 * ty + i] = ef;
-          }
-        }
-      }
-      __syncthreads();
-      if (GS) {
-        // gs = R1^T g over the units in order: thread -> atoms 4 ty .. + 3, inputs KPT tx .. + KPT - 1
-        float gq[4][KPT];
-#pragma unroll
-        for (int i = 0; i < 4; ++i)
-#pragma unroll
-          for (int j = 0; j < KPT; ++j) gq[i][j] = 0.0f;
-#pragma unroll 4
-        for (int o = 0; o < FH; ++o) {
-          const float gv[4] = {sG[(4 * ty) * GP + o], sG[(4 * ty + 1) * GP + o], sG[(4 * ty + 2) * GP + o],
-                               sG[(4 * ty + 3) * GP + o]};
-          float r[KPT];
-#pragma unroll
-          for (int j = 0; j < KPT; j += 4) {
-            const float4 q = *reinterpret_cast<const float4*>(sR1 + o * F + KPT * tx + j);
-            r[j] = q.x; r[j + 1] = q.y; r[j + 2] = q.z; r[j + 3] = q.w;
-          }
-#pragma unroll
-          for (int i = 0; i < 4; ++i)
-#pragma unroll
-            for (int j = 0; j < KPT; ++j) gq[i][j] = fmaf(gv[i], r[j], gq[i][j]);
-        }
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-          const int64_t ai = a0 + 4 * ty + i;
-          if (ai < n)
-#pragma unroll
-            for (int j = 0; j < KPT; j += 4)
-              *reinterpret_cast<float4*>(GS + ai * F + KPT * tx + j) =
-                  make_float4(gq[i][j], gq[i][j + 1], gq[i][j + 2], gq[i][j + 3]);
-        }
-      }
-      __syncthreads();   // the next tile overwrites s^T and g
+  const int64_t G = (int64_t)gridDim.x * TA;
+  for (int64_t a0 = (int64_t)blockIdx.x * TA; a0 < n; a0 += G) {
+    for (int idx = tid; idx < TA * F4; idx += NT) {
+      const int a = idx % TA, k4 = idx / TA;
+      float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+      if (a0 + a < n) v = reinterpret_cast<const float4*>(S + (a0 + a) * F)[k4];
+      sST[(4 * k4 + 0) * TA + a] = v.x;
+      sST[(4 * k4 + 1) * TA + a] = v.y;
+      sST[(4 * k4 + 2) * TA + a] = v.z;
+      sST[(4 * k4 + 3) * TA + a] = v.w;
     }
-    if (tid < 256 && base + tid < n) {
+    __syncthreads();
+    {
+      float h[4][OPT];
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int j = 0; j < OPT; ++j) h[i][j] = 0.0f;
+#pragma unroll 4
+      for (int k = 0; k < F; ++k) {
+        const float4 sa = *reinterpret_cast<const float4*>(sST + k * TA + 4 * ty);
+        float r[OPT];
+        if constexpr (OPT == 4) {
+          const float4 q = *reinterpret_cast<const float4*>(sR1T + k * FH + 4 * tx);
+          r[0] = q.x; r[1] = q.y; r[2] = q.z; r[3] = q.w;
+        } else {
+          const float2 q = *reinterpret_cast<const float2*>(sR1T + k * FH + 2 * tx);
+          r[0] = q.x; r[1] = q.y;
+        }
+        const float sv[4] = {sa.x, sa.y, sa.z, sa.w};
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+#pragma unroll
+          for (int j = 0; j < OPT; ++j) h[i][j] = fmaf(sv[i], r[j], h[i][j]);
+      }
+      // energy terms of this thread's units, each product split exactly (FMA) and added into a
+      // float-float pair (TwoSum), the pairs of the 16 threads of an atom combined in a fixed
+      // tree: the terms can largely cancel, and this keeps ~44 bits of their sum without the
+      // FP64 pipe; g = w e_scale R2 silu'(h) goes to the g tile
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const int64_t ai = a0 + 4 * ty + i;
+        const float wi = ai < n && ew ? ew[ai] : 1.0f;
+        float es = 0.0f, ec = 0.0f;
+#pragma unroll
+        for (int j = 0; j < OPT; ++j) {
+          const int o = OPT * tx + j;
+          const float hk = h[i][j] + (d1 ? d1[o] : 0.0f);
+          const float sl = silu_f(hk), pr = __fmul_rn(sR2[o], sl);
+          ff_add(es, ec, pr, __fmaf_rn(sR2[o], sl, -pr));
+          if (GS) sG[(4 * ty + i) * GP + o] = ai < n ? wi * (e_scale * sR2[o] * dsilu_f(hk)) : 0.0f;
+        }
+#pragma unroll
+        for (int off = 1; off < 16; off <<= 1) {
+          const float os = __shfl_xor_sync(0xffffffffu, es, off), oc = __shfl_xor_sync(0xffffffffu, ec, off);
+          ff_add(es, ec, os, oc);
+        }
+        if (tx == 0) {
+          double e = ((double)es + (double)ec + (double)d2[0]) * (double)e_scale;
+          e *= (double)wi;
+          const float ef = ai < n ? (float)e : 0.0f;
+          if (ai < n && e_atom) e_atom[ai] = ef;
+          sE[4 * ty + i] = ef;
+        }
+      }
+    }
+    __syncthreads();
+    if (GS) {
+      // gs = R1^T g over the units in order: thread -> atoms 4 ty .. + 3, inputs KPT tx .. + KPT - 1
+      float gq[4][KPT];
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int j = 0; j < KPT; ++j) gq[i][j] = 0.0f;
+#pragma unroll 4
+      for (int o = 0; o < FH; ++o) {
+        const float gv[4] = {sG[(4 * ty) * GP + o], sG[(4 * ty + 1) * GP + o], sG[(4 * ty + 2) * GP + o],
+                             sG[(4 * ty + 3) * GP + o]};
+        float r[KPT];
+#pragma unroll
+        for (int j = 0; j < KPT; j += 4) {
+          const float4 q = *reinterpret_cast<const float4*>(sR1 + o * F + KPT * tx + j);
+          r[j] = q.x; r[j + 1] = q.y; r[j + 2] = q.z; r[j + 3] = q.w;
+        }
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+#pragma unroll
+          for (int j = 0; j < KPT; ++j) gq[i][j] = fmaf(gv[i], r[j], gq[i][j]);
+      }
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const int64_t ai = a0 + 4 * ty + i;
+        if (ai < n)
+#pragma unroll
+          for (int j = 0; j < KPT; j += 4)
+            *reinterpret_cast<float4*>(GS + ai * F + KPT * tx + j) =
+                make_float4(gq[i][j], gq[i][j + 1], gq[i][j + 2], gq[i][j + 3]);
+      }
+    }
+    if (tid < TA && a0 + tid < n) {
       const double x = (double)sE[tid], t = acc + x;   // Neumaier
       comp += fabs(acc) >= fabs(x) ? (acc - t) + x : (x - t) + acc;
       acc = t;
     }
+    __syncthreads();   // the next tile overwrites s^T, g and the energies
   }
   double v = acc + comp;
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  if ((tid & 31) == 0 && tid < 256) sbuf[tid >> 5] = v;
+  if ((tid & 31) == 0 && tid < TA) sbuf[tid >> 5] = v;
   __syncthreads();
   if (tid == 0) {
     double sum = 0.0;
-    for (int w = 0; w < 8; ++w) sum += sbuf[w];
+    for (int w = 0; w < TA / 32; ++w) sum += sbuf[w];
     partials[blockIdx.x] = sum;
   }
 }
 
-template <int F>
+template <int F, int TA>
 static size_t readout_fused_smem() {
-  return sizeof(float) * ((size_t)2 * F * (F / 2) + (size_t)F * 128 + (size_t)128 * (F / 2 + 4) + 256 + F / 2);
+  return sizeof(float) * ((size_t)2 * F * (F / 2) + (size_t)F * TA + (size_t)TA * (F / 2 + 4) + TA + F / 2);
+}
+
+template <int F, int TA>
+static void launch_readout_fused(cudaStream_t st, const ModelW& m, int64_t n, const float* S_T, const float* ew, float* gs,
+                                 float* e_atom, double* partials, int n_partials) {
+  static const cudaError_t attr = cudaFuncSetAttribute(
+      k_readout_fused<F, TA>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)readout_fused_smem<F, TA>());
+  (void)attr;
+  LaunchScope ls_(st);
+  k_readout_fused<F, TA><<<n_partials, 4 * TA, readout_fused_smem<F, TA>(), st>>>(n, m.e_scale, S_T, m.R1, m.R1t, m.d1, m.R2,
+                                                                                 m.d2, ew, gs, e_atom, partials);
 }
 
 // F_i = sum_{e in row i} (hedge[rev e] - hedge[e]);  virial partials = sum_e r_e (x) hedge[e]
@@ -1235,20 +1248,11 @@ static void readout_fwd_bwd(cudaStream_t st, const ModelW& m, int64_t n, const f
                             bool need_grad, float* const* B, float* e_atom, double* partials, int n_partials) {
   const int F = m.F, Fh = F / 2;
   if (readout_is_fused(F)) {
-    LaunchScope ls_(st);
     float* gs = need_grad ? B[B_GS] : nullptr;
-    static bool attr = false;
-    if (!attr) {
-      cudaFuncSetAttribute(k_readout_fused<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)readout_fused_smem<128>());
-      cudaFuncSetAttribute(k_readout_fused<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)readout_fused_smem<64>());
-      attr = true;
-    }
-    if (F == 128)
-      k_readout_fused<128><<<n_partials, 512, readout_fused_smem<128>(), st>>>(n, m.e_scale, S_T, m.R1, m.R1t, m.d1,
-                                                                               m.R2, m.d2, ew, gs, e_atom, partials);
-    else
-      k_readout_fused<64><<<n_partials, 512, readout_fused_smem<64>(), st>>>(n, m.e_scale, S_T, m.R1, m.R1t, m.d1,
-                                                                             m.R2, m.d2, ew, gs, e_atom, partials);
+    const bool small = n <= 152 * 128;
+    auto go = F == 128 ? (small ? launch_readout_fused<128, 32> : launch_readout_fused<128, 128>)
+                       : (small ? launch_readout_fused<64, 32> : launch_readout_fused<64, 128>);
+    go(st, m, n, S_T, ew, gs, e_atom, partials, n_partials);
     return;
   }
   gemm<EPI_BIAS>(st, n, Fh, F, S_T, F, m.R1t, m.d1, nullptr, 0, B[B_H3], Fh);
