@@ -241,6 +241,14 @@ bool edge_tc_supported(int F, int K);
 int edge_bwd_tc(cudaStream_t st, const ModelW& m, int t, int accumulate, int64_t n, const int32_t* arow,
                 const int32_t* acol, const float4* ar, const float* PHI, float* GPHI, __nv_bfloat16* GP3b,
                 float4* hedge, int* status, const int32_t* aend, const float* G4, const __half* PHIh = nullptr);
+// edge_fp32.cu: the message step and its adjoint on CUDA cores in FP32.  wst (may be null): per-edge
+// filters and their distance derivatives, written by the message step, read by the adjoint
+void edge_msg_f32(cudaStream_t st, const ModelW& m, int t, int64_t n, const int32_t* arow, const int32_t* acol,
+                  const float4* ar, const float* PHI, const float* S, const float* V, float* SM, float* VM,
+                  __nv_bfloat16* VMb, float* wst);
+void edge_adj_f32(cudaStream_t st, const ModelW& m, int t, int accumulate, int64_t n, const int32_t* arow,
+                  const int32_t* acol, const float4* ar, const float* PHI, const float* Gsm, const float* Gvm,
+                  float* GPHI, float4* hedge, const float* wst);
 // edge_mma.cu: the message step as a tensor-core contraction over each receiver's edges
 // (F = 128, K < 32): gathered FP16 message rows x per-edge basis, FP32 filter weights after it.
 bool edge_mma_supported(int F, int K);

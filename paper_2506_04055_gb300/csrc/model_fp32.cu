@@ -17,12 +17,11 @@
 // GB300 layout: atoms are cell-sorted so neighbour gathers hit L2; per atom the gathered
 // message table is PHI = [phi_s | psi_0 | psi_1 | psi_2 | phi_vs | phi_vv] with
 // psi_a = v_a * phi_vv pre-multiplied once per atom (5F gathered floats per edge instead of 6F).
-// Edge kernels run one group of F threads per receiver row (thread = feature channel), so the
-// segmented sum over a receiver's CSR row stays in registers: no atomics.  The adjoint of the
-// message step runs sender-side: the row of atom j visits every edge whose sender is j (the
-// list holds both directions and the filter depends only on |r|), gathering the receivers'
-// gradients; per-edge position gradients go to hedge[e] and the forces are assembled from
-// hedge and the reverse-edge index, again without atomics.
+// The edge kernels (edge_fp32.cu) keep the segmented sum over a receiver's CSR row in registers: no
+// atomics.  The adjoint of the message step runs sender-side: the row of atom j visits every edge
+// whose sender is j (the list holds both directions and the filter depends only on |r|), gathering
+// the receivers' gradients; per-edge position gradients go to hedge[e] and the forces are assembled
+// from hedge and the reverse-edge index, again without atomics.
 #include "ctd_internal.cuh"
 #include "../../include/painn.h"
 
@@ -567,288 +566,6 @@ __global__ void k_phi_bwd_psi(int64_t n, int F, const float* __restrict__ GPSI, 
   st4(GP3b + i * 3 * F + F + f, gpvv);
 }
 
-// ================================================================================ edge kernels
-__device__ __forceinline__ void group_sync(int id, int nthreads) {
-  asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(nthreads) : "memory");
-}
-
-// Forward message: one group of F threads per receiver row.  Edges of the row are staged
-// F at a time (geometry, f_c, radial basis) in shared memory; thread f then accumulates
-// channel f of s and of the three components of v over the staged edges.
-//
-// STORE: the kernel also writes, per edge e and channel c in (s, vv, vs), the cutoff-scaled
-// filter W_c,e = f_c (Wf rbf + bf) and its distance derivative dW_c,e/dd, as
-// wst[e][6F] = [W_s | W_vv | W_vs | dW_s | dW_vv | dW_vs], so that the adjoint reads them
-// instead of recomputing the basis and the filter.
-template <int KP, bool STORE>
-__global__ __launch_bounds__(256) void k_edge_fwd(int64_t n, int F, int K, float rc,
-                                                  const int32_t* __restrict__ arow, const int32_t* __restrict__ acol,
-                                                  const float4* __restrict__ ar, const float* __restrict__ PHI,
-                                                  const float* __restrict__ S, const float* __restrict__ V,
-                                                  const float* __restrict__ Wf, const float* __restrict__ bf,
-                                                  float* __restrict__ SM, float* __restrict__ VM,
-                                                  __nv_bfloat16* __restrict__ VMb, float* __restrict__ wst,
-                                                  int v_zero) {
-  extern __shared__ __align__(16) float sm[];
-  constexpr int KD = STORE ? KP : 0;            // derivative basis staged only when storing
-  const int G = blockDim.x / F;                 // groups per block
-  const int g = threadIdx.x / F, f = threadIdx.x % F;
-  float* rbs = sm + (size_t)g * F * (KP + KD);                                   // [F edges][KP]
-  float* drbs = rbs + (size_t)F * KP;                                            // [F edges][KD]
-  float4* geo = reinterpret_cast<float4*>(sm + (size_t)G * F * (KP + KD)) + (size_t)g * F;  // (u, f_c)
-  float* dfcs = reinterpret_cast<float*>(sm + (size_t)G * F * (KP + KD + 4)) + (size_t)g * F;
-  int* js = reinterpret_cast<int*>(sm + (size_t)G * F * (KP + KD + 4 + (STORE ? 1 : 0))) + (size_t)g * F;
-
-  float w_s[KP], w_vv[KP], w_vs[KP];
-#pragma unroll
-  for (int k = 0; k < KP; ++k) {
-    w_s[k] = Wf[(size_t)f * KP + k];
-    w_vv[k] = Wf[(size_t)(F + f) * KP + k];
-    w_vs[k] = Wf[(size_t)(2 * F + f) * KP + k];
-  }
-  const float b_s = bf[f], b_vv = bf[F + f], b_vs = bf[2 * F + f];
-  const float inv_rc = 1.0f / rc, sig = rc / (float)(K - 1), inv2s2 = 1.0f / (2.0f * sig * sig);
-  const float inv_s2 = 1.0f / (sig * sig);
-  const int64_t ngroups = (int64_t)gridDim.x * G;
-
-  for (int64_t i = (int64_t)blockIdx.x * G + g; i < n; i += ngroups) {
-    const int a0 = arow[i], a1 = arow[i + 1];
-    float as = 0.f, av0 = 0.f, av1 = 0.f, av2 = 0.f;
-    for (int c0 = a0; c0 < a1; c0 += F) {
-      const int cnt = min(F, a1 - c0);
-      group_sync(1 + g, F);
-      if (f < cnt) {
-        float4 r = ar[c0 + f];
-        float d = r.w, id = 1.0f / d;
-        float fc = 0.5f * (cospif(d * inv_rc) + 1.0f);
-        geo[f] = make_float4(r.x * id, r.y * id, r.z * id, fc);
-        if (STORE) dfcs[f] = -0.5f * 3.14159265358979f * inv_rc * sinpif(d * inv_rc);
-        js[f] = acol[c0 + f];
-#pragma unroll
-        for (int k = 0; k < KP; ++k) {
-          float mu = (float)k * sig, t = d - mu;
-          const float v = k < K ? expf(-t * t * inv2s2) : 0.0f;
-          rbs[f * KP + k] = v;
-          if (STORE) drbs[f * KP + k] = -v * t * inv_s2;
-        }
-      }
-      group_sync(1 + g, F);
-      for (int t = 0; t < cnt; ++t) {
-        const float4 ge = geo[t];
-        const float* rb = rbs + t * KP;
-        float ws = b_s, wvv = b_vv, wvs = b_vs;
-#pragma unroll
-        for (int k = 0; k < KP; k += 4) {
-          float4 q = *reinterpret_cast<const float4*>(rb + k);
-          ws = fmaf(w_s[k], q.x, ws); ws = fmaf(w_s[k + 1], q.y, ws);
-          ws = fmaf(w_s[k + 2], q.z, ws); ws = fmaf(w_s[k + 3], q.w, ws);
-          wvv = fmaf(w_vv[k], q.x, wvv); wvv = fmaf(w_vv[k + 1], q.y, wvv);
-          wvv = fmaf(w_vv[k + 2], q.z, wvv); wvv = fmaf(w_vv[k + 3], q.w, wvv);
-          wvs = fmaf(w_vs[k], q.x, wvs); wvs = fmaf(w_vs[k + 1], q.y, wvs);
-          wvs = fmaf(w_vs[k + 2], q.z, wvs); wvs = fmaf(w_vs[k + 3], q.w, wvs);
-        }
-        // v_zero (first layer, v = 0): the psi channels v_a phi_vv are zero and not gathered
-        const float* p = PHI + (int64_t)js[t] * 6 * F;
-        const float ps = p[f], pvs = p[4 * F + f];
-        const float y0 = v_zero ? 0.f : p[F + f], y1 = v_zero ? 0.f : p[2 * F + f], y2 = v_zero ? 0.f : p[3 * F + f];
-        if (STORE) {
-          const float* drb = drbs + t * KP;
-          float dws = 0.f, dwvv = 0.f, dwvs = 0.f;
-#pragma unroll
-          for (int k = 0; k < KP; ++k) {
-            dws = fmaf(w_s[k], drb[k], dws);
-            dwvv = fmaf(w_vv[k], drb[k], dwvv);
-            dwvs = fmaf(w_vs[k], drb[k], dwvs);
-          }
-          const float fc = ge.w, dfc = dfcs[t];
-          float* o = wst + (int64_t)(c0 + t) * 6 * F + f;
-          o[0] = ws * fc;
-          o[F] = wvv * fc;
-          o[2 * F] = wvs * fc;
-          o[3 * F] = fc * dws + dfc * ws;
-          o[4 * F] = fc * dwvv + dfc * wvv;
-          o[5 * F] = fc * dwvs + dfc * wvs;
-        }
-        ws *= ge.w; wvv *= ge.w; wvs *= ge.w;
-        as = fmaf(ps, ws, as);
-        const float tvs = pvs * wvs;
-        av0 = fmaf(y0, wvv, fmaf(ge.x, tvs, av0));
-        av1 = fmaf(y1, wvv, fmaf(ge.y, tvs, av1));
-        av2 = fmaf(y2, wvv, fmaf(ge.z, tvs, av2));
-      }
-    }
-    SM[i * F + f] = S[i * F + f] + as;
-    VM[i * 3 * F + f] = V[i * 3 * F + f] + av0;
-    VM[i * 3 * F + F + f] = V[i * 3 * F + F + f] + av1;
-    VM[i * 3 * F + 2 * F + f] = V[i * 3 * F + 2 * F + f] + av2;
-    if (VMb) {
-      VMb[i * 3 * F + f] = __float2bfloat16_rn(VM[i * 3 * F + f]);
-      VMb[i * 3 * F + F + f] = __float2bfloat16_rn(VM[i * 3 * F + F + f]);
-      VMb[i * 3 * F + 2 * F + f] = __float2bfloat16_rn(VM[i * 3 * F + 2 * F + f]);
-    }
-  }
-}
-
-// Reduce four per-thread values over a warp; lane 8*q ends up with the sum of value q.
-__device__ __forceinline__ float warp_reduce4(float v0, float v1, float v2, float v3, int lane) {
-  // xor 16: lanes < 16 keep (v0, v1), lanes >= 16 keep (v2, v3)
-  bool hi = lane & 16;
-  float s0 = hi ? v0 : v2, s1 = hi ? v1 : v3;
-  float k0 = hi ? v2 : v0, k1 = hi ? v3 : v1;
-  k0 += __shfl_xor_sync(0xffffffffu, s0, 16);
-  k1 += __shfl_xor_sync(0xffffffffu, s1, 16);
-  // xor 8: lanes with bit 3 clear keep k0, set keep k1
-  bool b8 = lane & 8;
-  float s = b8 ? k0 : k1, k = b8 ? k1 : k0;
-  k += __shfl_xor_sync(0xffffffffu, s, 8);
-  k += __shfl_xor_sync(0xffffffffu, k, 4);
-  k += __shfl_xor_sync(0xffffffffu, k, 2);
-  k += __shfl_xor_sync(0xffffffffu, k, 1);
-  return k;   // lane 0: v0, lane 8: v1, lane 16: v2, lane 24: v3
-}
-
-// Adjoint of the message step, sender-side.  Row j holds edges e' = (j <- i); its reverse
-// (i <- j) carried phi_j, v_j into receiver i with direction u_rev = -u_e'.  Thread f gathers
-// (gsm_i, gvm_i) and accumulates d/dphi_s,j, d/dpsi_j,a, d/dphi_vs,j over the row; per edge the
-// partial d/dd and d/du_rev are reduced over the F channels and turned into
-// hedge[e'] = dU/dr_(i<-j).
-//
-// STORED: the filter and its distance derivative come from wst (written by k_edge_fwd<.., true>
-// for the same edge, whose distance equals its reverse's) instead of being recomputed.
-template <int KP, bool STORED>
-__global__ __launch_bounds__(256) void k_edge_bwd(int64_t n, int F, int K, float rc, int accumulate,
-                                                  const int32_t* __restrict__ arow, const int32_t* __restrict__ acol,
-                                                  const float4* __restrict__ ar, const float* __restrict__ PHI,
-                                                  const float* __restrict__ Gsm, const float* __restrict__ Gvm,
-                                                  const float* __restrict__ Wf, const float* __restrict__ bf,
-                                                  float* __restrict__ GPHI, float4* __restrict__ hedge,
-                                                  const float* __restrict__ wst) {
-  extern __shared__ __align__(16) float sm[];
-  constexpr int KB = STORED ? 0 : KP;   // basis staged only when recomputing
-  const int G = blockDim.x / F;
-  const int g = threadIdx.x / F, f = threadIdx.x % F, lane = threadIdx.x & 31, wig = f >> 5;
-  const int NW = F / 32;
-  float* rbs = sm + (size_t)g * F * (2 * KB + 8 + 4 * NW);     // [F][KB] rbf, [F][KB] drbf
-  float* drbs = rbs + F * KB;
-  float4* geo = reinterpret_cast<float4*>(drbs + F * KB);       // (u, d)
-  float4* gfc = geo + F;                                        // (f_c, f_c', -, -)
-  float* red = reinterpret_cast<float*>(gfc + F);               // [F edges][NW][4]
-  int* js = reinterpret_cast<int*>(sm + (size_t)G * F * (2 * KB + 8 + 4 * NW)) + (size_t)g * F;
-
-  float w_s[KB > 0 ? KB : 1], w_vv[KB > 0 ? KB : 1], w_vs[KB > 0 ? KB : 1];
-#pragma unroll
-  for (int k = 0; k < KB; ++k) {
-    w_s[k] = Wf[(size_t)f * KP + k];
-    w_vv[k] = Wf[(size_t)(F + f) * KP + k];
-    w_vs[k] = Wf[(size_t)(2 * F + f) * KP + k];
-  }
-  const float b_s = bf[f], b_vv = bf[F + f], b_vs = bf[2 * F + f];
-  const float inv_rc = 1.0f / rc, sig = rc / (float)(K - 1), inv2s2 = 1.0f / (2.0f * sig * sig);
-  const float inv_s2 = 1.0f / (sig * sig);
-  const int64_t ngroups = (int64_t)gridDim.x * G;
-
-  for (int64_t j = (int64_t)blockIdx.x * G + g; j < n; j += ngroups) {
-    const float* pj = PHI + j * 6 * F;
-    const float ps = pj[f], y0 = pj[F + f], y1 = pj[2 * F + f], y2 = pj[3 * F + f], pvs = pj[4 * F + f];
-    float gps = 0.f, gy0 = 0.f, gy1 = 0.f, gy2 = 0.f, gpvs = 0.f;
-    const int a0 = arow[j], a1 = arow[j + 1];
-    for (int c0 = a0; c0 < a1; c0 += F) {
-      const int cnt = min(F, a1 - c0);
-      group_sync(1 + g, F);
-      if (f < cnt) {
-        float4 r = ar[c0 + f];
-        float d = r.w, id = 1.0f / d;
-        float fc = 0.5f * (cospif(d * inv_rc) + 1.0f);
-        float dfc = -0.5f * 3.14159265358979f * inv_rc * sinpif(d * inv_rc);
-        geo[f] = make_float4(r.x * id, r.y * id, r.z * id, d);
-        gfc[f] = make_float4(fc, dfc, 0.f, 0.f);
-        js[f] = acol[c0 + f];
-#pragma unroll
-        for (int k = 0; k < KB; ++k) {
-          float t = d - (float)k * sig;
-          float rb = k < K ? expf(-t * t * inv2s2) : 0.0f;
-          rbs[f * KP + k] = rb;
-          drbs[f * KP + k] = -rb * t * inv_s2;
-        }
-      }
-      group_sync(1 + g, F);
-      for (int t = 0; t < cnt; ++t) {
-        const float4 ge = geo[t];
-        float Ws, Wvv, Wvs, pd_s, pd_vv, pd_vs;   // filter and dW/dd per channel (f_c folded in)
-        if (STORED) {
-          const float* w = wst + (int64_t)(c0 + t) * 6 * F + f;
-          Ws = w[0]; Wvv = w[F]; Wvs = w[2 * F];
-          pd_s = w[3 * F]; pd_vv = w[4 * F]; pd_vs = w[5 * F];
-        } else {
-          const float4 fcv = gfc[t];
-          const float* rb = rbs + t * KP;
-          const float* drb = drbs + t * KP;
-          float ws = b_s, wvv = b_vv, wvs = b_vs, dws = 0.f, dwvv = 0.f, dwvs = 0.f;
-#pragma unroll
-          for (int k = 0; k < KB; k += 4) {
-            float4 q = *reinterpret_cast<const float4*>(rb + k);
-            float4 dq = *reinterpret_cast<const float4*>(drb + k);
-            float qa[4] = {q.x, q.y, q.z, q.w}, da[4] = {dq.x, dq.y, dq.z, dq.w};
-#pragma unroll
-            for (int u = 0; u < 4; ++u) {
-              ws = fmaf(w_s[k + u], qa[u], ws);
-              wvv = fmaf(w_vv[k + u], qa[u], wvv);
-              wvs = fmaf(w_vs[k + u], qa[u], wvs);
-              dws = fmaf(w_s[k + u], da[u], dws);
-              dwvv = fmaf(w_vv[k + u], da[u], dwvv);
-              dwvs = fmaf(w_vs[k + u], da[u], dwvs);
-            }
-          }
-          const float fc = fcv.x, dfc = fcv.y;
-          Ws = ws * fc; Wvv = wvv * fc; Wvs = wvs * fc;
-          pd_s = fc * dws + dfc * ws; pd_vv = fc * dwvv + dfc * wvv; pd_vs = fc * dwvs + dfc * wvs;
-        }
-        const int64_t i = js[t];
-        const float gs = Gsm[i * F + f];
-        const float gv0 = Gvm[i * 3 * F + f], gv1 = Gvm[i * 3 * F + F + f], gv2 = Gvm[i * 3 * F + 2 * F + f];
-        gps = fmaf(gs, Ws, gps);
-        gy0 = fmaf(gv0, Wvv, gy0);
-        gy1 = fmaf(gv1, Wvv, gy1);
-        gy2 = fmaf(gv2, Wvv, gy2);
-        // u_rev = -u
-        const float q = -(gv0 * ge.x + gv1 * ge.y + gv2 * ge.z);
-        gpvs = fmaf(q, Wvs, gpvs);
-        const float gWs = gs * ps, gWvv = gv0 * y0 + gv1 * y1 + gv2 * y2, gWvs = q * pvs;
-        float pd = gWs * pd_s + gWvv * pd_vv + gWvs * pd_vs;
-        const float tv = pvs * Wvs;
-        float r = warp_reduce4(pd, gv0 * tv, gv1 * tv, gv2 * tv, lane);
-        if ((lane & 7) == 0) red[(t * NW + wig) * 4 + (lane >> 3)] = r;
-      }
-      group_sync(1 + g, F);
-      if (f < cnt) {
-        float pd = 0.f, gu0 = 0.f, gu1 = 0.f, gu2 = 0.f;
-        for (int w = 0; w < NW; ++w) {
-          const float* rr = red + (f * NW + w) * 4;
-          pd += rr[0]; gu0 += rr[1]; gu1 += rr[2]; gu2 += rr[3];
-        }
-        const float4 ge = geo[f];
-        const float ux = -ge.x, uy = -ge.y, uz = -ge.z, id = 1.0f / ge.w;
-        const float gdu = gu0 * ux + gu1 * uy + gu2 * uz;
-        float4 h = make_float4(pd * ux + (gu0 - gdu * ux) * id, pd * uy + (gu1 - gdu * uy) * id,
-                               pd * uz + (gu2 - gdu * uz) * id, 0.f);
-        if (accumulate) {
-          float4 o = hedge[c0 + f];
-          h.x += o.x; h.y += o.y; h.z += o.z;
-        }
-        hedge[c0 + f] = h;
-      }
-    }
-    if (GPHI) {
-      float* o = GPHI + j * 5 * F;
-      o[f] = gps;
-      o[F + f] = gy0;
-      o[2 * F + f] = gy1;
-      o[3 * F + f] = gy2;
-      o[4 * F + f] = gpvs;
-    }
-  }
-}
-
 // ================================================================================ readout, forces
 // h3 = R1 s + d1 (done by the GEMM); U_i = e_scale (R2 . silu(h3) + d2);
 // G3 = w_i e_scale R2 * silu'(h3) (seed of the backward pass); per-block FP64 partials of
@@ -1154,71 +871,6 @@ __global__ void k_forces(int64_t n, const int32_t* __restrict__ arow, const floa
 // ================================================================================ driver
 static inline unsigned blocks_for(int64_t work) { return (unsigned)((work + kThreads - 1) / kThreads); }
 
-template <int KP>
-static void edge_fwd_kp(cudaStream_t st, const ModelW& m, int t, int64_t n, const int32_t* arow,
-                        const int32_t* acol, const float4* ar, const float* PHI, const float* S, const float* V,
-                        float* SM, float* VM, __nv_bfloat16* VMb, float* wst) {
-  const int v_zero = t == 0;   // the first layer's v is the embedding's zero
-  const int F = m.F, G = kThreads / F;
-  const int KD = wst ? KP : 0;
-  size_t smem = (size_t)G * F * (KP + KD + 4 + (wst ? 1 : 0)) * sizeof(float) + (size_t)G * F * sizeof(int);
-  int64_t blocks = (n + G - 1) / G;
-  if (blocks > 152 * 16) blocks = 152 * 16;
-  if (blocks < 1) blocks = 1;
-  LaunchScope ls_(st);
-  if (wst)
-    k_edge_fwd<KP, true><<<(unsigned)blocks, kThreads, smem, st>>>(n, F, m.K, m.rc, arow, acol, ar, PHI, S, V,
-                                                                   m.L[t].Wf, m.L[t].bf, SM, VM, VMb, wst, v_zero);
-  else
-    k_edge_fwd<KP, false><<<(unsigned)blocks, kThreads, smem, st>>>(n, F, m.K, m.rc, arow, acol, ar, PHI, S, V,
-                                                                    m.L[t].Wf, m.L[t].bf, SM, VM, VMb, nullptr, v_zero);
-}
-
-template <int KP>
-static void edge_bwd_kp(cudaStream_t st, const ModelW& m, int t, int accumulate, int64_t n, const int32_t* arow,
-                        const int32_t* acol, const float4* ar, const float* PHI, const float* Gsm,
-                        const float* Gvm, float* GPHI, float4* hedge, const float* wst) {
-  const int F = m.F, G = kThreads / F, NW = F / 32;
-  const int KB = wst ? 0 : KP;
-  size_t smem = (size_t)G * F * (2 * KB + 8 + 4 * NW) * sizeof(float) + (size_t)G * F * sizeof(int);
-  int64_t blocks = (n + G - 1) / G;
-  if (blocks > 152 * 16) blocks = 152 * 16;
-  if (blocks < 1) blocks = 1;
-  LaunchScope ls_(st);
-  if (wst)
-    k_edge_bwd<KP, true><<<(unsigned)blocks, kThreads, smem, st>>>(n, F, m.K, m.rc, accumulate, arow, acol, ar, PHI,
-                                                                   Gsm, Gvm, m.L[t].Wf, m.L[t].bf, GPHI, hedge, wst);
-  else
-    k_edge_bwd<KP, false><<<(unsigned)blocks, kThreads, smem, st>>>(n, F, m.K, m.rc, accumulate, arow, acol, ar, PHI,
-                                                                    Gsm, Gvm, m.L[t].Wf, m.L[t].bf, GPHI, hedge, nullptr);
-}
-
-#define CTD_KP_DISPATCH(KPV, CALL) \
-  switch (KPV) {                   \
-    case 4: CALL(4); break;        \
-    case 8: CALL(8); break;        \
-    case 12: CALL(12); break;      \
-    case 16: CALL(16); break;      \
-    case 20: CALL(20); break;      \
-    case 24: CALL(24); break;      \
-    case 28: CALL(28); break;      \
-    default: CALL(32); break;      \
-  }
-
-void edge_smem_setup() {
-  static bool done = false;
-  if (done) return;
-  done = true;
-#define CTD_SET_SMEM(K_)                                                                              \
-  cudaFuncSetAttribute(k_edge_fwd<K_, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024); \
-  cudaFuncSetAttribute(k_edge_fwd<K_, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);  \
-  cudaFuncSetAttribute(k_edge_bwd<K_, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024); \
-  cudaFuncSetAttribute(k_edge_bwd<K_, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
-  CTD_SET_SMEM(4) CTD_SET_SMEM(8) CTD_SET_SMEM(12) CTD_SET_SMEM(16) CTD_SET_SMEM(20) CTD_SET_SMEM(24)
-  CTD_SET_SMEM(28) CTD_SET_SMEM(32)
-#undef CTD_SET_SMEM
-}
-
 // Buffers (all float, sized by the caller; see api.cu for the list and shapes).
 enum BufId {
   B_S0 = 0,                        // s, one buffer for every layer (ids B_S0 + t unused)
@@ -1317,7 +969,6 @@ void model_forward_backward_fp32(cudaStream_t st, const ModelW& m, int64_t n, co
                                  float* force_s, double* virial_partials, int n_virial_partials,
                                  float* e_atom, int* status, float* wstore, int64_t wstore_layer_floats,
                                  const float* ew) {
-  edge_smem_setup();
   StageGuard node_stage(STG_NODE);
   const int F = m.F, T = m.T;
   const unsigned nb = blocks_for(n * F), nb4 = blocks_for(n * F / 4);   // nb4: four features per thread
@@ -1333,12 +984,10 @@ void model_forward_backward_fp32(cudaStream_t st, const ModelW& m, int64_t n, co
     if (n > 0) { LaunchScope ls_(st); k_phi_pack<<<nb, kThreads, 0, st>>>(n, F, T2, V, PHI); }
     // message
     float* wst = (wstore && need_grad) ? wstore + t * wstore_layer_floats : nullptr;
-#define CTD_FWD(KPV) edge_fwd_kp<KPV>(st, m, t, n, arow, acol, ar, PHI, S, V, SM, VM, nullptr, wst)
-    if (n > 0) {
+    {
       StageGuard sg(STG_EDGE_FWD);
-      CTD_KP_DISPATCH(m.KP, CTD_FWD)
+      edge_msg_f32(st, m, t, n, arow, acol, ar, PHI, S, V, SM, VM, nullptr, wst);
     }
-#undef CTD_FWD
     // update
     gemm<EPI_BIAS>(st, 3 * n, 2 * F, F, VM, F, L.UVt, nullptr, nullptr, 0, UV, 2 * F);
     if (n > 0) { LaunchScope ls_(st); k_update_pre<float><<<nb4, kThreads, 0, st>>>(n, F, m.eps, SM, UV, T1, nullptr); }
@@ -1375,12 +1024,10 @@ void model_forward_backward_fp32(cudaStream_t st, const ModelW& m, int64_t n, co
     // the first layer's inputs (embedding, v = 0) do not depend on positions: its edge adjoint
     // writes no phi gradients and the phi backward below it is skipped
     float* gphi = t > 0 ? GPHI : nullptr;
-#define CTD_BWD(KPV) edge_bwd_kp<KPV>(st, m, t, t != T - 1, n, arow, acol, ar, PHI, GSM, GVM, gphi, hedge, wst)
-    if (n > 0) {
+    {
       StageGuard sg(STG_EDGE_BWD);
-      CTD_KP_DISPATCH(m.KP, CTD_BWD)
+      edge_adj_f32(st, m, t, t != T - 1, n, arow, acol, ar, PHI, GSM, GVM, gphi, hedge, wst);
     }
-#undef CTD_BWD
     if (t == 0) break;
     // phi backward -> gradients w.r.t. the layer input (s_t, v_t)
     if (n > 0) { LaunchScope ls_(st); k_phi_bwd_pre<<<nb, kThreads, 0, st>>>(n, F, GPHI, PHI, nullptr, V, GVM, T2, GV, nullptr); }
@@ -1459,7 +1106,6 @@ int model_forward_backward_bf16(cudaStream_t st, const ModelW& m, int64_t n, con
                                 double* virial_partials, int n_virial_partials, float* e_atom, int* status,
                                 float* wstore, int64_t wstore_layer_floats, const int32_t* aend,
                                 const float* ew) {
-  edge_smem_setup();
   StageGuard node_stage(STG_NODE);
   const int F = m.F, T = m.T;
   const unsigned nb = blocks_for(n * F), nb4 = blocks_for(n * F / 4);   // nb4: four features per thread
@@ -1496,16 +1142,13 @@ int model_forward_backward_bf16(cudaStream_t st, const ModelW& m, int64_t n, con
     const float* Vin = (t == 0 && msg_mma) ? nullptr : V;   // null: v = 0, psi = 0
     bad |= gemm_bf16<4>(st, n, 3 * F, F, Bb[BB_A1], F, L.W2b, L.b2, Vin, 3 * F, PHI, 6 * F, nullptr, 0, status, PHIh);
     float* wst = (wstore && need_grad && !use_tc_bwd && !msg_mma) ? wstore + t * wstore_layer_floats : nullptr;
-#define CTD_FWD(KPV) edge_fwd_kp<KPV>(st, m, t, n, arow, acol, ar, PHI, S, V, SM, VM, Bb[BB_VM], wst)
     if (n > 0) {
       StageGuard sg(STG_EDGE_FWD);
-      if (msg_mma) {
+      if (msg_mma)
         bad |= edge_fwd_mma(st, m, t, n, arow, acol, ar, PHIh, S, Vin, SM, VM, Bb[BB_VM], status);
-      } else {
-        CTD_KP_DISPATCH(m.KP, CTD_FWD)
-      }
+      else
+        edge_msg_f32(st, m, t, n, arow, acol, ar, PHI, S, V, SM, VM, Bb[BB_VM], wst);
     }
-#undef CTD_FWD
     bad |= gemm_bf16<0>(st, 3 * n, 2 * F, F, Bb[BB_VM], F, L.UVb, nullptr, nullptr, 0, nullptr, 2 * F, nullptr, 0,
                         status, UV);
     if (n > 0) { LaunchScope ls_(st); k_update_pre<__half><<<nb4, kThreads, 0, st>>>(n, F, m.eps, SM, UV, nullptr, Bb[BB_Z]); }
@@ -1551,17 +1194,14 @@ int model_forward_backward_bf16(cudaStream_t st, const ModelW& m, int64_t n, con
     const float* wst = (wstore && !use_tc_bwd && !msg_mma) ? wstore + t * wstore_layer_floats : nullptr;
     // first layer: no phi gradients, no phi backward (its inputs do not depend on positions)
     float* gphi = t > 0 ? GPHI : nullptr;
-#define CTD_BWD(KPV) edge_bwd_kp<KPV>(st, m, t, t != T - 1, n, arow, acol, ar, PHI, GSM, GVM, gphi, hedge, wst)
     if (n > 0) {
       StageGuard sg(STG_EDGE_BWD);
-      if (use_tc_bwd) {
+      if (use_tc_bwd)
         bad |= edge_bwd_tc(st, m, t, t != T - 1, n, arow, acol, ar, PHI, gphi, gphi ? Bb[BB_GP3] : nullptr, hedge,
                            status, aend, G4, phi32 ? nullptr : PHIh);
-      } else {
-        CTD_KP_DISPATCH(m.KP, CTD_BWD)
-      }
+      else
+        edge_adj_f32(st, m, t, t != T - 1, n, arow, acol, ar, PHI, GSM, GVM, gphi, hedge, wst);
     }
-#undef CTD_BWD
     if (t == 0) break;
     if (n > 0) {
       LaunchScope ls_(st);
