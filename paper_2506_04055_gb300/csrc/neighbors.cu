@@ -9,9 +9,9 @@
 //                 slab index per direction, atom counts per cell
 //   scan + place  counting sort by cell; sort_cells makes the order within a cell ascending
 //                 in the caller's index, so the whole build is deterministic
-//   pair_search   one warp per atom, lanes over the atoms of each neighbour cell, the pair
-//                 test in FP64 with __dmul_rn/__dadd_rn in the canonical order, warp-ballot
-//                 compaction; run twice (count, then fill at scanned offsets)
+//   pair_search   warps over the cells, lanes over (home atom, candidate) pairs of each neighbour
+//                 cell, an FP32 prefilter and the pair test in FP64 with __dmul_rn/__dadd_rn in the
+//                 canonical order, warp-ballot compaction; run twice (count, then fill at scanned offsets)
 //   reverse       rev[e] = index of (j <- i, -n) for e = (i <- j, n)
 // Per step:
 //   delta         d_i = x_i - x_ref,i (FP64 -> FP32) and the largest |d_i|^2 (skin trigger)
@@ -127,11 +127,16 @@ __device__ __forceinline__ uint32_t pack_img(int a, int b, int c) {
          ((uint32_t)(uint8_t)(int8_t)c << 16);
 }
 
-// One warp per cell of the grid: the cell's atoms (in groups of up to 32, the "home" atoms)
-// against the atoms of every neighbour cell, visited in a fixed order of slab offsets; within a
-// neighbour cell the candidates are in sorted order.  Each neighbour cell is staged in shared
-// memory (in pieces of up to kPsPiece atoms, image shift applied) and the lanes run over the
+// A warp takes home atoms of one cell of the grid (up to 32 at a time, or a fixed share of them: a
+// cell's atoms are dealt to nsub warps, 32 / nsub each) against the atoms of every neighbour cell,
+// visited in a fixed order of slab offsets; within a neighbour cell the candidates are in sorted
+// order.  The lanes work out the bounds and images of 32 neighbour cells at once; each
+// neighbour cell is staged in shared memory (in pieces of up to kPsPiece atoms, image shift applied),
+// the next piece's positions on their way meanwhile, and the lanes run over the
 // (home atom, candidate) pairs, so all 32 lanes work whatever the cell occupancy.
+// nsub: a grid of few cells left most SMs without a warp (5,997 atoms, 216 cells: 540 us per
+// pass); nsub grows until every SM has 16 warps.  More than one warp per cell stages the neighbour
+// cells once per warp, which costs large grids more than it gives.
 //
 // Every pair first takes an FP32 distance test against R2f, a threshold above R^2 by a bound on
 // the FP32 rounding of the positions, the image shift and the squared distance (computed on the
@@ -139,13 +144,13 @@ __device__ __forceinline__ uint32_t pack_img(int a, int b, int c) {
 // the cutoff.  The survivors (about one in seven) queue up per warp in the order they were found
 // and take the canonical FP64 test in batches of 32.  The pairs kept are those of the FP64 test
 // alone; each home atom's row lists them by neighbour cell, then candidate, and is written
-// through a per-atom cursor, so the fill is deterministic.
+// through a per-atom cursor, so the fill is deterministic and does not depend on nsub.
 constexpr int kPsQueue = 64;   // per-warp survivor queue (a batch of 32 plus one chunk)
 constexpr int kPsPiece = 64;   // neighbour atoms staged at a time
 constexpr int kPsWarps = kThreads / 32;
 
 template <bool FILL>
-__global__ void k_pair_search(int64_t ncells, const double* __restrict__ xs, const int32_t* __restrict__ cstart,
+__global__ void k_pair_search(int64_t ncells, int nsub, const double* __restrict__ xs, const int32_t* __restrict__ cstart,
                               CellGeom g, float r2f, int32_t* __restrict__ count, const int32_t* __restrict__ row_ptr,
                               int32_t* __restrict__ col, uint32_t* __restrict__ img,
                               float4* __restrict__ base) {
@@ -155,8 +160,8 @@ __global__ void k_pair_search(int64_t ncells, const double* __restrict__ xs, con
   __shared__ int32_t qj[kPsWarps][kPsQueue];
   __shared__ uint32_t qi[kPsWarps][kPsQueue];
   __shared__ int32_t qa[kPsWarps][kPsQueue];
-  const int64_t cw = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
-  const int lane = threadIdx.x & 31, wq = threadIdx.x >> 5;
+  const int64_t gw = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5, cw = gw / nsub;
+  const int lane = threadIdx.x & 31, wq = threadIdx.x >> 5, share = 32 / nsub;
   if (cw >= ncells) return;
   const unsigned lt = (1u << lane) - 1u;
   const int c0 = (int)(cw / ((int64_t)g.nc[1] * g.nc[2])), c1 = (int)((cw / g.nc[2]) % g.nc[1]),
@@ -165,8 +170,9 @@ __global__ void k_pair_search(int64_t ncells, const double* __restrict__ xs, con
   const int hs = cstart[hlin], he = cstart[hlin + 1];
   const float hf[9] = {(float)g.H[0], (float)g.H[1], (float)g.H[2], (float)g.H[3], (float)g.H[4],
                        (float)g.H[5], (float)g.H[6], (float)g.H[7], (float)g.H[8]};
-  for (int h0 = hs; h0 < he; h0 += 32) {
-    const int ga = he - h0 < 32 ? he - h0 : 32;
+  const int m1 = 2 * g.M[1] + 1, m2 = 2 * g.M[2] + 1, noff = (2 * g.M[0] + 1) * m1 * m2;
+  for (int h0 = hs + (int)(gw % nsub) * share; h0 < he; h0 += 32) {
+    const int ga = he - h0 < share ? he - h0 : share;
     if (lane < ga) {
       const int64_t i = h0 + lane;
       hx[wq][lane] = make_float4((float)xs[3 * i], (float)xs[3 * i + 1], (float)xs[3 * i + 2], 0.f);
@@ -210,67 +216,102 @@ __global__ void k_pair_search(int64_t ncells, const double* __restrict__ xs, con
       if (lane < nb && (peers & lt) == 0) cur[wq][a] += __popc(m & peers);   // one lane per home atom
       __syncwarp();
     };
-    for (int d0 = -g.M[0]; d0 <= g.M[0]; ++d0)
-      for (int d1 = -g.M[1]; d1 <= g.M[1]; ++d1)
-        for (int d2 = -g.M[2]; d2 <= g.M[2]; ++d2) {
-          int cc[3] = {c0 + d0, c1 + d1, c2 + d2};
-          int im[3], w[3];
-          for (int a = 0; a < 3; ++a) {
-            int q = cc[a] >= 0 ? cc[a] / g.nc[a] : -((-cc[a] + g.nc[a] - 1) / g.nc[a]);
-            im[a] = q;
-            w[a] = cc[a] - q * g.nc[a];
+    for (int o0 = 0; o0 < noff; o0 += 32) {
+      // lane l: bounds and image of neighbour cell o0 + l
+      int mbs = 0, mbe = 0;
+      uint32_t mpim = 0;
+      if (o0 + lane < noff) {
+        const int o = o0 + lane;
+        const int cc[3] = {c0 + o / (m1 * m2) - g.M[0], c1 + o / m2 % m1 - g.M[1], c2 + o % m2 - g.M[2]};
+        int im[3], w[3];
+        for (int a = 0; a < 3; ++a) {
+          const int q = cc[a] >= 0 ? cc[a] / g.nc[a] : -((-cc[a] + g.nc[a] - 1) / g.nc[a]);
+          im[a] = q;
+          w[a] = cc[a] - q * g.nc[a];
+        }
+        const int nlin = cell_linear(g, w[0], w[1], w[2]);
+        mbs = cstart[nlin];
+        mbe = cstart[nlin + 1];
+        mpim = pack_img(im[0], im[1], im[2]);
+      }
+      unsigned todo = __ballot_sync(0xffffffffu, mbe > mbs);   // non-empty cells not yet begun
+      int b0 = 0, be = 0, nb = 0;
+      uint32_t pim = 0;
+      double px[2][3];
+      // the next piece of up to kPsPiece atoms; its positions are loaded into px
+      auto advance = [&]() {
+        if (b0 + kPsPiece < be) {
+          b0 += kPsPiece;
+        } else if (todo) {
+          const int k = __ffs(todo) - 1;
+          todo &= todo - 1;
+          b0 = __shfl_sync(0xffffffffu, mbs, k);
+          be = __shfl_sync(0xffffffffu, mbe, k);
+          pim = __shfl_sync(0xffffffffu, mpim, k);
+        } else {
+          nb = 0;
+          return;
+        }
+        nb = be - b0 < kPsPiece ? be - b0 : kPsPiece;
+#pragma unroll
+        for (int h = 0; h < 2; ++h)
+          if (lane + 32 * h < nb)
+#pragma unroll
+            for (int c = 0; c < 3; ++c) px[h][c] = xs[3 * (int64_t)(b0 + lane + 32 * h) + c];
+      };
+      static_assert(kPsPiece == 64, "two atoms per lane");
+      advance();
+      while (nb > 0) {
+        const int cb0 = b0, cnb = nb;
+        const uint32_t cpim = pim;
+        const float i0 = (float)(int8_t)(cpim & 0xff), i1 = (float)(int8_t)((cpim >> 8) & 0xff), i2 = (float)(int8_t)((cpim >> 16) & 0xff);
+        float shf[3];
+        for (int c = 0; c < 3; ++c) shf[c] = fmaf(i0, hf[c], fmaf(i1, hf[3 + c], i2 * hf[6 + c]));
+        const bool zero_img = cpim == 0;
+#pragma unroll
+        for (int h = 0; h < 2; ++h)
+          if (lane + 32 * h < cnb)
+            nx[wq][lane + 32 * h] = make_float4((float)px[h][0] + shf[0], (float)px[h][1] + shf[1], (float)px[h][2] + shf[2], 0.f);
+        __syncwarp();
+        advance();
+        const int total = ga * cnb;
+        const float rnb = 1.0f / (float)cnb;
+        for (int p0 = 0; p0 < total; p0 += 32) {
+          const int p = p0 + lane;
+          bool pass = false;
+          int a = 0, bb = 0;
+          if (p < total) {
+            // p / cnb: p < 2048 and the quotient's distance from an integer is at least 1 / 128
+            a = (int)(((float)p + 0.5f) * rnb);
+            bb = p - a * cnb;
+            const float4 y = nx[wq][bb], x = hx[wq][a];
+            const float e0 = y.x - x.x, e1 = y.y - x.y, e2 = y.z - x.z;
+            pass = fmaf(e2, e2, fmaf(e1, e1, e0 * e0)) < r2f && !(zero_img && cb0 + bb == h0 + a);
           }
-          float shf[3];
-          for (int c = 0; c < 3; ++c)
-            shf[c] = fmaf((float)im[0], hf[c], fmaf((float)im[1], hf[3 + c], (float)im[2] * hf[6 + c]));
-          const bool zero_img = (im[0] == 0) && (im[1] == 0) && (im[2] == 0);
-          const uint32_t pim = pack_img(im[0], im[1], im[2]);
-          const int nlin = cell_linear(g, w[0], w[1], w[2]);
-          const int bs = cstart[nlin], be = cstart[nlin + 1];
-          for (int b0 = bs; b0 < be; b0 += kPsPiece) {
-            const int nb = be - b0 < kPsPiece ? be - b0 : kPsPiece;
-            for (int t = lane; t < nb; t += 32) {
-              const int64_t jj = b0 + t;
-              nx[wq][t] = make_float4((float)xs[3 * jj] + shf[0], (float)xs[3 * jj + 1] + shf[1],
-                                      (float)xs[3 * jj + 2] + shf[2], 0.f);
-            }
+          const unsigned m = __ballot_sync(0xffffffffu, pass);
+          if (pass) {
+            const int slot = qn + __popc(m & lt);
+            qj[wq][slot] = cb0 + bb;
+            qi[wq][slot] = cpim;
+            qa[wq][slot] = a;
+          }
+          qn += __popc(m);
+          __syncwarp();
+          if (qn >= 32) {
+            batch(32);
+            // move the overflow (at most 31 entries) to the front of the queue
+            int32_t mj = 0, ma = 0;
+            uint32_t mi = 0;
+            if (lane + 32 < qn) { mj = qj[wq][lane + 32]; mi = qi[wq][lane + 32]; ma = qa[wq][lane + 32]; }
             __syncwarp();
-            const int total = ga * nb;
-            for (int p0 = 0; p0 < total; p0 += 32) {
-              const int p = p0 + lane;
-              bool pass = false;
-              int a = 0, bb = 0;
-              if (p < total) {
-                a = p / nb;
-                bb = p - a * nb;
-                const float4 y = nx[wq][bb], x = hx[wq][a];
-                const float e0 = y.x - x.x, e1 = y.y - x.y, e2 = y.z - x.z;
-                pass = fmaf(e2, e2, fmaf(e1, e1, e0 * e0)) < r2f && !(zero_img && b0 + bb == h0 + a);
-              }
-              const unsigned m = __ballot_sync(0xffffffffu, pass);
-              if (pass) {
-                const int slot = qn + __popc(m & lt);
-                qj[wq][slot] = b0 + bb;
-                qi[wq][slot] = pim;
-                qa[wq][slot] = a;
-              }
-              qn += __popc(m);
-              __syncwarp();
-              if (qn >= 32) {
-                batch(32);
-                // move the overflow (at most 31 entries) to the front of the queue
-                int32_t mj = 0, ma = 0;
-                uint32_t mi = 0;
-                if (lane + 32 < qn) { mj = qj[wq][lane + 32]; mi = qi[wq][lane + 32]; ma = qa[wq][lane + 32]; }
-                __syncwarp();
-                if (lane + 32 < qn) { qj[wq][lane] = mj; qi[wq][lane] = mi; qa[wq][lane] = ma; }
-                qn -= 32;
-                __syncwarp();
-              }
-            }
-            __syncwarp();   // the piece is read before the next one overwrites it
+            if (lane + 32 < qn) { qj[wq][lane] = mj; qi[wq][lane] = mi; qa[wq][lane] = ma; }
+            qn -= 32;
+            __syncwarp();
           }
         }
+        __syncwarp();   // the piece is read before the next one overwrites it
+      }
+    }
     if (qn > 0) batch(qn);
     if (!FILL && lane < ga) count[h0 + lane] = cur[wq][lane];
     __syncwarp();
@@ -297,14 +338,16 @@ void launch_pair_search(cudaStream_t st, bool fill, int64_t n, const double* xw_
                         const int32_t* cell_start, const CellGeom& g, int32_t* count,
                         const int32_t* row_ptr, int32_t* col, uint32_t* img, float4* base) {
   if (n == 0) return;
-  const int64_t ncells = (int64_t)g.nc[0] * g.nc[1] * g.nc[2];   // one warp per grid cell
-  const int64_t threads = ncells * 32;
+  const int64_t ncells = (int64_t)g.nc[0] * g.nc[1] * g.nc[2];
+  int nsub = 1;   // warps per grid cell
+  while (nsub < 32 && ncells * nsub < 152 * 16) nsub *= 2;
+  const int64_t threads = ncells * nsub * 32;
   const unsigned blocks = (unsigned)((threads + kThreads - 1) / kThreads);
   const float r2f = prefilter_r2(g);
   if (fill)
-    { LaunchScope ls_(st); k_pair_search<true><<<blocks, kThreads, 0, st>>>(ncells, xw_s, cell_start, g, r2f, count, row_ptr, col, img, base); }
+    { LaunchScope ls_(st); k_pair_search<true><<<blocks, kThreads, 0, st>>>(ncells, nsub, xw_s, cell_start, g, r2f, count, row_ptr, col, img, base); }
   else
-    { LaunchScope ls_(st); k_pair_search<false><<<blocks, kThreads, 0, st>>>(ncells, xw_s, cell_start, g, r2f, count, row_ptr, col, img, base); }
+    { LaunchScope ls_(st); k_pair_search<false><<<blocks, kThreads, 0, st>>>(ncells, nsub, xw_s, cell_start, g, r2f, count, row_ptr, col, img, base); }
 }
 
 // ------------------------------------------------------------------------------- reverse edges
@@ -313,25 +356,61 @@ __device__ __forceinline__ uint32_t neg_img(uint32_t v) {
   return pack_img(-a, -b, -c);
 }
 
-// One warp per row i; for each edge e = (i <- j, n) the warp scans row j for (j <- i, -n).
+// One warp per row i; for each edge e = (i <- j, n) the warp scans row j for (j <- i, -n).  Two edges
+// at a time, up to 96 entries of each row in flight at once: one memory latency per two edges
+// instead of one per 32 entries of each.
 __global__ void k_reverse(int64_t n, const int32_t* __restrict__ rp, const int32_t* __restrict__ col,
                           const uint32_t* __restrict__ img, int32_t* __restrict__ rev, int* status) {
+  constexpr int NB = 3;
   int64_t i = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
   int lane = threadIdx.x & 31;
   if (i >= n) return;
-  for (int e = rp[i]; e < rp[i + 1]; ++e) {
-    int j = col[e];
-    uint32_t want = neg_img(img[e]);
-    int found = -1;
-    for (int b = rp[j]; b < rp[j + 1] && found < 0; b += 32) {
-      int k = b + lane;
-      bool hit = (k < rp[j + 1]) && col[k] == (int)i && img[k] == want;
-      unsigned m = __ballot_sync(0xffffffffu, hit);
-      if (m) found = b + __ffs(m) - 1;
+  const int r0 = rp[i], r1 = rp[i + 1];
+  for (int e0 = r0; e0 < r1; e0 += 32) {
+    // lane l: edge e0 + l, its wanted image and the bounds of its row
+    const int me = min(e0 + lane, r1 - 1);
+    const int mj = col[me];
+    const uint32_t mw = neg_img(img[me]);
+    const int mb = rp[mj], mend = rp[mj + 1];
+    int mine = -1;
+    const int cnt = min(32, r1 - e0);
+    for (int k = 0; k < cnt; k += 2) {
+      int b[2], end[2], c[2][NB];
+      uint32_t want[2], im[2][NB];
+#pragma unroll
+      for (int u = 0; u < 2; ++u) {
+        const int src = min(k + u, cnt - 1);
+        b[u] = __shfl_sync(0xffffffffu, mb, src);
+        end[u] = __shfl_sync(0xffffffffu, mend, src);
+        want[u] = __shfl_sync(0xffffffffu, mw, src);
+      }
+      int found[2] = {-1, -1};
+      while ((found[0] < 0 && b[0] < end[0]) || (found[1] < 0 && b[1] < end[1])) {
+#pragma unroll
+        for (int u = 0; u < 2; ++u)
+#pragma unroll
+          for (int q = 0; q < NB; ++q) {
+            const int x = b[u] + 32 * q + lane;
+            const bool in = found[u] < 0 && x < end[u];
+            c[u][q] = in ? col[x] : -1;
+            im[u][q] = in ? img[x] : 0u;
+          }
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+#pragma unroll
+          for (int q = 0; q < NB; ++q) {
+            const unsigned m = __ballot_sync(0xffffffffu, c[u][q] == (int)i && im[u][q] == want[u]);
+            if (m && found[u] < 0) found[u] = b[u] + 32 * q + __ffs(m) - 1;
+          }
+          b[u] += 32 * NB;
+        }
+      }
+      if (lane == k) mine = found[0];
+      if (lane == k + 1) mine = found[1];
     }
-    if (lane == 0) {
-      rev[e] = found;
-      if (found < 0) atomicOr(status, (int)ST_REV_MISSING);
+    if (lane < cnt) {
+      rev[e0 + lane] = mine;
+      if (mine < 0) atomicOr(status, (int)ST_REV_MISSING);
     }
   }
 }
