@@ -53,34 +53,53 @@ __global__ void k_concat_verlet(const RepDesc* __restrict__ reps, int32_t* __res
   }
 }
 
-// Per-replica reductions, one block per replica, fixed order (independent of the batch).
-// out[r*12 + 0] = sum of per-atom energies, [1] = kinetic energy (eV), [2] = max |d|^2,
-// [3..11] = virial.
-__global__ void k_rep_reduce(const int64_t* __restrict__ aoff, const int32_t* __restrict__ arow,
+// Per-replica sums: [0] per-atom energies, [1] kinetic energy (eV), [2] max |d|^2, [3..11] virial, in
+// FP64.  A replica's atoms are cut into slices of kSliceAtoms counted from its first atom; a block
+// sums one slice (a warp per atom's row, its edges over the lanes; each warp its rows in order, the lanes by a
+// shuffle tree, the warps in order), a second kernel a replica's slices in order, so a replica's
+// sums do not depend on the batch.  (One block per replica with a thread per row took 600 us for
+// replicas of up to 4,000 atoms, bound by the one SM that held the largest.)
+constexpr int kSliceAtoms = 64;
+// The first slice of the replica that begins at atom a0 and is the r-th of the batch: leaves room
+// for its ceil(atoms / kSliceAtoms) slices whatever the alignment of its bounds.
+__host__ __device__ __forceinline__ int64_t first_slice(int64_t a0, int64_t r) { return a0 / kSliceAtoms + r; }
+
+__global__ void k_rep_slices(int nres, const int64_t* __restrict__ aoff, const int32_t* __restrict__ arow,
                              const float* __restrict__ eatom, const double* __restrict__ mass,
                              const double* __restrict__ vel, const float4* __restrict__ delta,
                              const float4* __restrict__ ar, const float4* __restrict__ hedge, int with_virial,
                              double* __restrict__ out) {
   __shared__ double sh[12][kThreads / 32];
-  const int64_t a0 = aoff[blockIdx.x], a1 = aoff[blockIdx.x + 1];
+  int lo = 0, hi = nres - 1;   // the last replica whose first slice is not beyond this block's
+  while (lo < hi) {
+    const int mid = (lo + hi + 1) / 2;
+    if (first_slice(aoff[mid], mid) <= (int64_t)blockIdx.x) lo = mid;
+    else hi = mid - 1;
+  }
+  const int64_t a0 = aoff[lo] + ((int64_t)blockIdx.x - first_slice(aoff[lo], lo)) * kSliceAtoms;
+  const int64_t end = aoff[lo + 1], a1 = a0 + kSliceAtoms < end ? a0 + kSliceAtoms : end;
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   double acc[12];
   for (int q = 0; q < 12; ++q) acc[q] = 0.0;
   constexpr double kAccConv = 9.648533212331002e-3;
-  for (int64_t i = a0 + threadIdx.x; i < a1; i += blockDim.x) {
-    acc[0] += (double)eatom[i];
-    acc[1] += 0.5 * mass[i] * (vel[3 * i] * vel[3 * i] + vel[3 * i + 1] * vel[3 * i + 1] + vel[3 * i + 2] * vel[3 * i + 2]) /
-              kAccConv;
-    const float4 d = delta[i];
-    acc[2] = fmax(acc[2], (double)(d.x * d.x + d.y * d.y + d.z * d.z));
-    if (with_virial)
-      for (int e = arow[i]; e < arow[i + 1]; ++e) {
+  if (w < kSliceAtoms / 32) {   // per-atom terms: thread = atom of the slice
+    const int64_t i = a0 + threadIdx.x;
+    if (i < a1) {
+      acc[0] = (double)eatom[i];
+      acc[1] = 0.5 * mass[i] * (vel[3 * i] * vel[3 * i] + vel[3 * i + 1] * vel[3 * i + 1] + vel[3 * i + 2] * vel[3 * i + 2]) /
+               kAccConv;
+      const float4 d = delta[i];
+      acc[2] = (double)(d.x * d.x + d.y * d.y + d.z * d.z);
+    }
+  }
+  if (with_virial)
+    for (int64_t i = a0 + w; i < a1; i += kThreads / 32)
+      for (int e = arow[i] + lane; e < arow[i + 1]; e += 32) {
         const float4 r = ar[e], h = hedge[e];
         const float rr[3] = {r.x, r.y, r.z}, hh[3] = {h.x, h.y, h.z};
         for (int p = 0; p < 3; ++p)
           for (int q = 0; q < 3; ++q) acc[3 + 3 * p + q] += (double)rr[p] * (double)hh[q];
       }
-  }
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   for (int q = 0; q < 12; ++q) {
     double v = acc[q];
     for (int o = 16; o > 0; o >>= 1) {
@@ -92,10 +111,37 @@ __global__ void k_rep_reduce(const int64_t* __restrict__ aoff, const int32_t* __
   __syncthreads();
   if (threadIdx.x < 12) {
     const int q = threadIdx.x;
-    double v = q == 2 ? 0.0 : 0.0;
+    double v = 0.0;
     for (int k = 0; k < kThreads / 32; ++k) v = q == 2 ? fmax(v, sh[q][k]) : v + sh[q][k];
     out[(int64_t)blockIdx.x * 12 + q] = v;
   }
+}
+
+// out[r*12 + q]: the sums of replica r over its slices; one block of 12 warps per replica, warp = q.
+__global__ void k_rep_sum(const int64_t* __restrict__ aoff, const double* __restrict__ slices, double* __restrict__ out) {
+  const int64_t r = blockIdx.x, n = aoff[r + 1] - aoff[r], ns = (n + kSliceAtoms - 1) / kSliceAtoms;
+  const double* s = slices + first_slice(aoff[r], r) * 12;
+  const int q = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  double v = 0.0;
+  for (int64_t k = lane; k < ns; k += 32) v = q == 2 ? fmax(v, s[k * 12 + q]) : v + s[k * 12 + q];
+  for (int o = 16; o > 0; o >>= 1) {
+    const double x = __shfl_xor_sync(0xffffffffu, v, o);
+    v = q == 2 ? fmax(v, x) : v + x;
+  }
+  if (lane == 0) out[r * 12 + q] = v;
+}
+
+static void rep_reduce(cudaStream_t st, int64_t natoms, int64_t nres, const int64_t* aoff, const int32_t* arow, const float* eatom,
+                       const double* mass, const double* vel, const float4* delta, const float4* ar, const float4* hedge,
+                       int with_virial, double* slices, double* out) {
+  if (nres == 0) return;
+  {
+    LaunchScope ls_(st);
+    k_rep_slices<<<(unsigned)first_slice(natoms, nres), kThreads, 0, st>>>((int)nres, aoff, arow, eatom, mass, vel, delta, ar,
+                                                                           hedge, with_virial, slices);
+  }
+  LaunchScope ls_(st);
+  k_rep_sum<<<(unsigned)nres, 12 * 32, 0, st>>>(aoff, slices, out);
 }
 
 // Velocity-Verlet halves for replicas whose flag says "integrating" (a replica's first step
@@ -178,7 +224,7 @@ struct ctd_server {
   std::unordered_map<int64_t, Replica*> reps;
   size_t resident_est = 0;
   // batch bookkeeping (device)
-  DBuf rep_table, rep_off, rep_of_atom, rep_flags, rep_out;
+  DBuf rep_table, rep_off, rep_of_atom, rep_flags, rep_out, rep_slices;
   // thermostats of the resident replicas (when any has one): parameters, chain states,
   // kinetic energy after the last step, velocity factors, chain energies
   DBuf rep_np, rep_chain, rep_ke, rep_g, rep_eth;
@@ -198,7 +244,7 @@ struct ctd_server {
   uint64_t gkey = 0, last_key = 0;
   int64_t graph_kernels = 0, steps_graph = 0, steps_eager = 0, captures = 0;
   std::vector<DBuf*> bufs() {
-    return {&rep_table, &rep_off, &rep_of_atom, &rep_flags, &rep_out, &rep_np, &rep_chain, &rep_ke, &rep_g, &rep_eth, &st_x, &st_xref, &st_v, &st_m, &st_z, &st_f,
+    return {&rep_table, &rep_off, &rep_of_atom, &rep_flags, &rep_out, &rep_slices, &rep_np, &rep_chain, &rep_ke, &rep_g, &rep_eth, &st_x, &st_xref, &st_v, &st_m, &st_z, &st_f,
             &b_xw, &b_wrap, &b_cell, &b_ccount, &b_cstart, &b_cursor, &b_tmp, &b_perm, &b_inv, &b_xws, &b_xnew,
             &b_count, &b_img, &b_scan, &b_i32, &b_d3};
   }
@@ -385,6 +431,7 @@ int repack(ctd_server* s, const std::vector<Replica*>& next) {
   ENSURE(c, s->rep_of_atom, sizeof(int32_t) * N1);
   ENSURE(c, s->rep_flags, sizeof(int32_t) * (R > 0 ? R : 1));
   ENSURE(c, s->rep_out, sizeof(double) * 12 * (R > 0 ? R : 1));
+  ENSURE(c, s->rep_slices, sizeof(double) * 12 * (first_slice(N, R) + 1));
   std::vector<int64_t> offs(R + 1, 0);
   for (int64_t k = 0; k < R; ++k) offs[k + 1] = offs[k] + next[k]->n;
   CUDA_OK(c, cudaMemcpyAsync(s->rep_off.p, offs.data(), sizeof(int64_t) * (R + 1), cudaMemcpyHostToDevice, st));
@@ -523,13 +570,9 @@ int step_device(ctd_server* s, int64_t nres) {
                                                P<int32_t>(s->rep_of_atom), P<int32_t>(s->rep_flags),
                                                P<double>(c->md_v));
   }
-  {
-    LaunchScope ls_(st);
-    k_rep_reduce<<<(unsigned)nres, kThreads, 0, st>>>(P<int64_t>(s->rep_off), P<int32_t>(c->arow),
-                                                     P<float>(c->eatom), P<double>(c->md_m), P<double>(c->md_v),
-                                                     P<float4>(c->delta), P<float4>(c->ar), P<float4>(c->hedge), 1,
-                                                     P<double>(s->rep_out));
-  }
+  rep_reduce(st, N, nres, P<int64_t>(s->rep_off), P<int32_t>(c->arow), P<float>(c->eatom), P<double>(c->md_m),
+             P<double>(c->md_v), P<float4>(c->delta), P<float4>(c->ar), P<float4>(c->hedge), 1, P<double>(s->rep_slices),
+             P<double>(s->rep_out));
   if (s->any_nvt) {
     launch_rep_nhc_half(st, (int)nres, P<NhcParams>(s->rep_np), 0.5 * s->dt, P<double>(s->rep_out) + 1, 12,
                         P<int32_t>(s->rep_flags), P<double>(s->rep_chain), kChainStride, P<double>(s->rep_g),
@@ -725,10 +768,8 @@ int ctd_serve_step(ctd_server* s, int32_t* n_resident, int32_t* n_admitted, int3
   {
     StageGuard sg(STG_PRUNE);
     launch_delta(st, N, P<double>(c->x_s), P<double>(c->xref_s), P<float4>(c->delta), P<unsigned int>(c->maxd));
-    LaunchScope ls_(st);
-    k_rep_reduce<<<(unsigned)nres, kThreads, 0, st>>>(P<int64_t>(s->rep_off), nullptr, P<float>(c->force_s),
-                                                     P<double>(c->md_m), P<double>(c->md_v), P<float4>(c->delta),
-                                                     nullptr, nullptr, 0, P<double>(s->rep_out));
+    rep_reduce(st, N, nres, P<int64_t>(s->rep_off), nullptr, P<float>(c->force_s), P<double>(c->md_m), P<double>(c->md_v),
+               P<float4>(c->delta), nullptr, nullptr, 0, P<double>(s->rep_slices), P<double>(s->rep_out));
   }
   std::vector<double> ro(12 * nres);
   CUDA_OK(c, cudaMemcpyAsync(ro.data(), s->rep_out.p, sizeof(double) * 12 * nres, cudaMemcpyDeviceToHost, st));
