@@ -208,7 +208,7 @@ int build_from_device_positions(ctd_ctx* c, int64_t n, const double H[9], double
   launch_sort_cells(st, c->ncell, P<int32_t>(c->cell_start), P<int32_t>(c->tmp_idx), P<int32_t>(c->perm));
   launch_gather_sorted(st, n, P<int32_t>(c->perm), P<double>(c->xw), P<double>(c->x_user), nullptr,
                        P<double>(c->xw_s), P<double>(c->xref_s), nullptr, P<int32_t>(c->inv_perm));
-  launch_pair_search(st, false, n, P<double>(c->xw_s), P<int32_t>(c->cell_start), c->geom, P<int32_t>(c->count),
+  launch_pair_search(st, false, n, P<double>(c->xw_s), P<float4>(c->xw), P<int32_t>(c->cell_start), c->geom, P<int32_t>(c->count),
                      nullptr, nullptr, nullptr, nullptr);
   launch_exclusive_scan(st, n, P<int32_t>(c->count), P<int32_t>(c->vrow), c->scan_tmp.p);
   int32_t total = 0;
@@ -222,7 +222,7 @@ int build_from_device_positions(ctd_ctx* c, int64_t n, const double H[9], double
   ENSURE(c, c->vbase, sizeof(float4) * e1);
   ENSURE(c, c->vrev, sizeof(int32_t) * e1);
   ENSURE(c, c->v2a, sizeof(int32_t) * e1);
-  launch_pair_search(st, true, n, P<double>(c->xw_s), P<int32_t>(c->cell_start), c->geom, P<int32_t>(c->count),
+  launch_pair_search(st, true, n, P<double>(c->xw_s), P<float4>(c->xw), P<int32_t>(c->cell_start), c->geom, P<int32_t>(c->count),
                      P<int32_t>(c->vrow), P<int32_t>(c->vcol), P<uint32_t>(c->vimg), P<float4>(c->vbase));
   launch_reverse(st, n, P<int32_t>(c->vrow), P<int32_t>(c->vcol), P<uint32_t>(c->vimg), P<int32_t>(c->vrev),
                  P<int>(c->status));

@@ -184,7 +184,8 @@ void launch_sort_cells(cudaStream_t st, int64_t ncell, const int32_t* cell_start
 void launch_gather_sorted(cudaStream_t st, int64_t n, const int32_t* perm, const double* xw,
                           const double* x_user, const int32_t* species_user, double* xw_s,
                           double* xref_s, int32_t* species_s, int32_t* inv_perm);
-void launch_pair_search(cudaStream_t st, bool fill, int64_t n, const double* xw_s,
+// xf: scratch of n float4 (16-byte aligned), kept from the count pass (fill false) to the fill pass
+void launch_pair_search(cudaStream_t st, bool fill, int64_t n, const double* xw_s, float4* xf,
                         const int32_t* cell_start, const CellGeom& g, int32_t* count,
                         const int32_t* row_ptr, int32_t* col, uint32_t* img, float4* base);
 void launch_reverse(cudaStream_t st, int64_t n, const int32_t* row_ptr, const int32_t* col,

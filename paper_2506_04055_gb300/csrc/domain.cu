@@ -401,7 +401,7 @@ int build_domain(ctd_domains* D, Dom& M, const double* xcand, const int32_t* csr
                                                    cown + off, P<int32_t>(D->bsrc) + off,
                                                    P<double>(D->bshift) + 3 * off, P<uint8_t>(D->bown) + off);
   }
-  launch_pair_search(st, false, n, P<double>(D->b_xws), P<int32_t>(D->b_cstart), M.geom, P<int32_t>(D->b_count),
+  launch_pair_search(st, false, n, P<double>(D->b_xws), P<float4>(D->b_xw), P<int32_t>(D->b_cstart), M.geom, P<int32_t>(D->b_count),
                      nullptr, nullptr, nullptr, nullptr);
   launch_exclusive_scan(st, n, P<int32_t>(D->b_count), P<int32_t>(M.vrow), D->b_scan.p);
   int32_t total = 0;
@@ -413,7 +413,7 @@ int build_domain(ctd_domains* D, Dom& M, const double* xcand, const int32_t* csr
   ENSURE(c, M.vbase, sizeof(float4) * e1);
   ENSURE(c, M.vrev, sizeof(int32_t) * e1);
   ENSURE(c, D->b_img, sizeof(uint32_t) * e1);
-  launch_pair_search(st, true, n, P<double>(D->b_xws), P<int32_t>(D->b_cstart), M.geom, P<int32_t>(D->b_count),
+  launch_pair_search(st, true, n, P<double>(D->b_xws), P<float4>(D->b_xw), P<int32_t>(D->b_cstart), M.geom, P<int32_t>(D->b_count),
                      P<int32_t>(M.vrow), P<int32_t>(M.vcol), P<uint32_t>(D->b_img), P<float4>(M.vbase));
   launch_reverse(st, n, P<int32_t>(M.vrow), P<int32_t>(M.vcol), P<uint32_t>(D->b_img), P<int32_t>(M.vrev),
                  P<int>(c->status));

@@ -134,6 +134,8 @@ __device__ __forceinline__ uint32_t pack_img(int a, int b, int c) {
 // neighbour cell is staged in shared memory (in pieces of up to kPsPiece atoms, image shift applied),
 // the next piece's positions on their way meanwhile, and the lanes run over the
 // (home atom, candidate) pairs, so all 32 lanes work whatever the cell occupancy.
+// FP64 runs at a sixty-fourth of the FP32 rate here, conversions included: the prefilter reads an FP32
+// copy of the positions (xf), and the canonical test takes its image shift from a table.
 // nsub: a grid of few cells left most SMs without a warp (5,997 atoms, 216 cells: 540 us per
 // pass); nsub grows until every SM has 16 warps.  More than one warp per cell stages the neighbour
 // cells once per warp, which costs large grids more than it gives.
@@ -150,10 +152,12 @@ constexpr int kPsPiece = 64;   // neighbour atoms staged at a time
 constexpr int kPsWarps = kThreads / 32;
 
 template <bool FILL>
-__global__ void k_pair_search(int64_t ncells, int nsub, const double* __restrict__ xs, const int32_t* __restrict__ cstart,
+__global__ void k_pair_search(int64_t ncells, int nsub, const double* __restrict__ xs,
+                              const float4* __restrict__ xf, const int32_t* __restrict__ cstart,
                               CellGeom g, float r2f, int32_t* __restrict__ count, const int32_t* __restrict__ row_ptr,
                               int32_t* __restrict__ col, uint32_t* __restrict__ img,
                               float4* __restrict__ base) {
+  __shared__ double shift1[27][3];
   __shared__ float4 hx[kPsWarps][32];          // home atoms (FP32)
   __shared__ float4 nx[kPsWarps][kPsPiece];    // neighbour piece (FP32, image shift applied)
   __shared__ int32_t cur[kPsWarps][32];        // per home atom: pairs kept so far
@@ -162,6 +166,13 @@ __global__ void k_pair_search(int64_t ncells, int nsub, const double* __restrict
   __shared__ int32_t qa[kPsWarps][kPsQueue];
   const int64_t gw = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5, cw = gw / nsub;
   const int lane = threadIdx.x & 31, wq = threadIdx.x >> 5, share = 32 / nsub;
+  // the image shifts by -1, 0, 1 cells in FP64, in the canonical order of operations
+  if (threadIdx.x < 27) {
+    const double m0 = (double)((int)threadIdx.x / 9 - 1), m1 = (double)((int)threadIdx.x / 3 % 3 - 1), m2 = (double)((int)threadIdx.x % 3 - 1);
+    for (int c = 0; c < 3; ++c)
+      shift1[threadIdx.x][c] = __dadd_rn(__dadd_rn(__dmul_rn(m0, g.H[c]), __dmul_rn(m1, g.H[3 + c])), __dmul_rn(m2, g.H[6 + c]));
+  }
+  __syncthreads();
   if (cw >= ncells) return;
   const unsigned lt = (1u << lane) - 1u;
   const int c0 = (int)(cw / ((int64_t)g.nc[1] * g.nc[2])), c1 = (int)((cw / g.nc[2]) % g.nc[1]),
@@ -174,8 +185,7 @@ __global__ void k_pair_search(int64_t ncells, int nsub, const double* __restrict
   for (int h0 = hs + (int)(gw % nsub) * share; h0 < he; h0 += 32) {
     const int ga = he - h0 < share ? he - h0 : share;
     if (lane < ga) {
-      const int64_t i = h0 + lane;
-      hx[wq][lane] = make_float4((float)xs[3 * i], (float)xs[3 * i + 1], (float)xs[3 * i + 2], 0.f);
+      hx[wq][lane] = xf[h0 + lane];
       cur[wq][lane] = 0;
     }
     __syncwarp();
@@ -194,9 +204,14 @@ __global__ void k_pair_search(int64_t ncells, int nsub, const double* __restrict
         const int64_t i = h0 + a;
         const int im0 = (int8_t)(pim & 0xff), im1 = (int8_t)((pim >> 8) & 0xff), im2 = (int8_t)((pim >> 16) & 0xff);
         double sh[3];
-        for (int c = 0; c < 3; ++c)
-          sh[c] = __dadd_rn(__dadd_rn(__dmul_rn((double)im0, g.H[c]), __dmul_rn((double)im1, g.H[3 + c])),
-                            __dmul_rn((double)im2, g.H[6 + c]));
+        if (abs(im0) <= 1 && abs(im1) <= 1 && abs(im2) <= 1) {
+          const double* t = shift1[(im0 + 1) * 9 + (im1 + 1) * 3 + im2 + 1];
+          for (int c = 0; c < 3; ++c) sh[c] = t[c];
+        } else {
+          for (int c = 0; c < 3; ++c)
+            sh[c] = __dadd_rn(__dadd_rn(__dmul_rn((double)im0, g.H[c]), __dmul_rn((double)im1, g.H[3 + c])),
+                              __dmul_rn((double)im2, g.H[6 + c]));
+        }
         dv0 = __dadd_rn(__dsub_rn(xs[3 * (int64_t)j], xs[3 * i]), sh[0]);
         dv1 = __dadd_rn(__dsub_rn(xs[3 * (int64_t)j + 1], xs[3 * i + 1]), sh[1]);
         dv2 = __dadd_rn(__dsub_rn(xs[3 * (int64_t)j + 2], xs[3 * i + 2]), sh[2]);
@@ -237,7 +252,7 @@ __global__ void k_pair_search(int64_t ncells, int nsub, const double* __restrict
       unsigned todo = __ballot_sync(0xffffffffu, mbe > mbs);   // non-empty cells not yet begun
       int b0 = 0, be = 0, nb = 0;
       uint32_t pim = 0;
-      double px[2][3];
+      float4 px[2];
       // the next piece of up to kPsPiece atoms; its positions are loaded into px
       auto advance = [&]() {
         if (b0 + kPsPiece < be) {
@@ -255,9 +270,7 @@ __global__ void k_pair_search(int64_t ncells, int nsub, const double* __restrict
         nb = be - b0 < kPsPiece ? be - b0 : kPsPiece;
 #pragma unroll
         for (int h = 0; h < 2; ++h)
-          if (lane + 32 * h < nb)
-#pragma unroll
-            for (int c = 0; c < 3; ++c) px[h][c] = xs[3 * (int64_t)(b0 + lane + 32 * h) + c];
+          if (lane + 32 * h < nb) px[h] = xf[b0 + lane + 32 * h];
       };
       static_assert(kPsPiece == 64, "two atoms per lane");
       advance();
@@ -271,7 +284,7 @@ __global__ void k_pair_search(int64_t ncells, int nsub, const double* __restrict
 #pragma unroll
         for (int h = 0; h < 2; ++h)
           if (lane + 32 * h < cnb)
-            nx[wq][lane + 32 * h] = make_float4((float)px[h][0] + shf[0], (float)px[h][1] + shf[1], (float)px[h][2] + shf[2], 0.f);
+            nx[wq][lane + 32 * h] = make_float4(px[h].x + shf[0], px[h].y + shf[1], px[h].z + shf[2], 0.f);
         __syncwarp();
         advance();
         const int total = ga * cnb;
@@ -334,7 +347,13 @@ static float prefilter_r2(const CellGeom& g) {
   return std::nextafter((float)t, INFINITY);
 }
 
-void launch_pair_search(cudaStream_t st, bool fill, int64_t n, const double* xw_s,
+// xf: scratch of n float4, written by the count pass, read by both
+__global__ void k_positions_f32(int64_t n, const double* __restrict__ xs, float4* __restrict__ xf) {
+  const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  if (i < n) xf[i] = make_float4((float)xs[3 * i], (float)xs[3 * i + 1], (float)xs[3 * i + 2], 0.f);
+}
+
+void launch_pair_search(cudaStream_t st, bool fill, int64_t n, const double* xw_s, float4* xf,
                         const int32_t* cell_start, const CellGeom& g, int32_t* count,
                         const int32_t* row_ptr, int32_t* col, uint32_t* img, float4* base) {
   if (n == 0) return;
@@ -344,10 +363,14 @@ void launch_pair_search(cudaStream_t st, bool fill, int64_t n, const double* xw_
   const int64_t threads = ncells * nsub * 32;
   const unsigned blocks = (unsigned)((threads + kThreads - 1) / kThreads);
   const float r2f = prefilter_r2(g);
+  if (!fill) {
+    LaunchScope ls_(st);
+    k_positions_f32<<<(unsigned)((n + kThreads - 1) / kThreads), kThreads, 0, st>>>(n, xw_s, xf);
+  }
   if (fill)
-    { LaunchScope ls_(st); k_pair_search<true><<<blocks, kThreads, 0, st>>>(ncells, nsub, xw_s, cell_start, g, r2f, count, row_ptr, col, img, base); }
+    { LaunchScope ls_(st); k_pair_search<true><<<blocks, kThreads, 0, st>>>(ncells, nsub, xw_s, xf, cell_start, g, r2f, count, row_ptr, col, img, base); }
   else
-    { LaunchScope ls_(st); k_pair_search<false><<<blocks, kThreads, 0, st>>>(ncells, nsub, xw_s, cell_start, g, r2f, count, row_ptr, col, img, base); }
+    { LaunchScope ls_(st); k_pair_search<false><<<blocks, kThreads, 0, st>>>(ncells, nsub, xw_s, xf, cell_start, g, r2f, count, row_ptr, col, img, base); }
 }
 
 // ------------------------------------------------------------------------------- reverse edges

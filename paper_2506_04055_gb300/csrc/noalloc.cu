@@ -247,7 +247,7 @@ extern "C" int ctd_neighbors_noalloc(int64_t n, const double* positions, const d
   launch_place(st, n, cellid, cstart, cursor, tmp);
   launch_sort_cells(st, ncell, cstart, tmp, perm);
   launch_gather_sorted(st, n, perm, xw, positions, nullptr, xw_s, xref, nullptr, inv);
-  launch_pair_search(st, false, n, xw_s, cstart, g, count, nullptr, nullptr, nullptr, nullptr);
+  launch_pair_search(st, false, n, xw_s, reinterpret_cast<float4*>(xw), cstart, g, count, nullptr, nullptr, nullptr, nullptr);
   int stv[2] = {0, 0};
   if (total_may_overflow) {
     // the row offsets are an int32 scan: total the per-atom counts in int64 first

@@ -320,7 +320,7 @@ int build_replica(ctd_server* s, Replica& R) {
   launch_sort_cells(st, R.ncell, P<int32_t>(s->b_cstart), P<int32_t>(s->b_tmp), P<int32_t>(s->b_perm));
   launch_gather_sorted(st, n, P<int32_t>(s->b_perm), P<double>(s->b_xw), X, nullptr, P<double>(s->b_xws),
                        P<double>(s->b_xnew), nullptr, P<int32_t>(s->b_inv));
-  launch_pair_search(st, false, n, P<double>(s->b_xws), P<int32_t>(s->b_cstart), R.geom, P<int32_t>(s->b_count),
+  launch_pair_search(st, false, n, P<double>(s->b_xws), P<float4>(s->b_xw), P<int32_t>(s->b_cstart), R.geom, P<int32_t>(s->b_count),
                      nullptr, nullptr, nullptr, nullptr);
   launch_exclusive_scan(st, n, P<int32_t>(s->b_count), P<int32_t>(R.vrow), s->b_scan.p);
   int32_t total = 0;
@@ -332,7 +332,7 @@ int build_replica(ctd_server* s, Replica& R) {
   ENSURE(c, R.vbase, sizeof(float4) * e1);
   ENSURE(c, R.vrev, sizeof(int32_t) * e1);
   ENSURE(c, s->b_img, sizeof(uint32_t) * e1);
-  launch_pair_search(st, true, n, P<double>(s->b_xws), P<int32_t>(s->b_cstart), R.geom, P<int32_t>(s->b_count),
+  launch_pair_search(st, true, n, P<double>(s->b_xws), P<float4>(s->b_xw), P<int32_t>(s->b_cstart), R.geom, P<int32_t>(s->b_count),
                      P<int32_t>(R.vrow), P<int32_t>(R.vcol), P<uint32_t>(s->b_img), P<float4>(R.vbase));
   launch_reverse(st, n, P<int32_t>(R.vrow), P<int32_t>(R.vcol), P<uint32_t>(s->b_img), P<int32_t>(R.vrev),
                  P<int>(c->status));
