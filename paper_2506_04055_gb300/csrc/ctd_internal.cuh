@@ -151,7 +151,8 @@ int local_forward_backward(cudaStream_t st, const LocalW& w, int64_t n, int64_t 
 void launch_forces(cudaStream_t st, int64_t n, const int32_t* arow, const float4* ar, const int32_t* arev,
                    const float4* hedge, float* force, double* vpart, int n_vpart, int* status);
 // out = A B (+ epilogue) with the FP32 SIMT GEMM: epi 0 bias (may be null), 1 bias + silu into
-// out2, 2 out = A B + aux (aux and out must not overlap), 3 out = (A B) * silu'(aux).
+// out2, 2 out = A B + aux (aux and out must not overlap), 3 out = (A B) * silu'(aux),
+// 4 out = (A B + aux) * silu'(out2) (out2 read only).
 void gemm_f32(cudaStream_t st, int epi, int64_t M, int N, int K, const float* A, int lda, const float* B,
               const float* bias, const float* aux, int ldaux, float* out, int ldo, float* out2, int ldo2);
 
@@ -232,7 +233,7 @@ void launch_check_finite(cudaStream_t st, int64_t n, const double* a, int* statu
 // EPI 0 bias, 1 bias + SiLU (bf16 copy gets the SiLU; outh: FP16 copy of the argument), 2 + aux,
 // 3 * SiLU'(aux), 4 PHI packing,
 // 5 + aux written as the interleaved (aux2, rows 3i..3i+2) quads of the adjoint's G4,
-// 6 * SiLU'(auxh), the argument stored in FP16.
+// 6 * SiLU'(auxh), the argument stored in FP16, 7 (+ aux) * SiLU'(aux2), aux2 [M][N].
 bool gemm_bf16_supported(int N, int K);
 bool make_tmap_bf16(CUtensorMap* m, const void* base, int64_t rows, int64_t cols, int64_t ld, int box_rows);
 // edge_tc.cu: tensor-core edge adjoint (F = 128, K <= 31); G4 = the receivers' (gsm, gvm)

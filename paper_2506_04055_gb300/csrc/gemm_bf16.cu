@@ -261,10 +261,19 @@ __global__ void __launch_bounds__(64 + 32 * epi_warps<EPI>(), 1) k_gemm_bf16(con
             gh[j] = m < p.M ? __ldg(reinterpret_cast<const uint2*>(p.auxh + m * p.ldaux + c0 + cc)) : make_uint2(0u, 0u);
           }
         }
+        float4 g7[EPI == 7 ? 4 : 1], z7[EPI == 7 ? 4 : 1];   // EPI 7: two operands, four rows in flight at a time
 #pragma unroll
         for (int j = 0; j < 8; ++j) {
           const int r = cr + 4 * j;
           const int64_t m = m0 + r;
+          if (EPI == 7 && j % 4 == 0) {
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+              const int64_t mq = m + 4 * q < p.M ? m + 4 * q : p.M - 1;
+              g7[q] = __ldg(reinterpret_cast<const float4*>(p.aux + mq * p.ldaux + c0 + cc));
+              z7[q] = __ldg(reinterpret_cast<const float4*>(p.aux2 + mq * N + c0 + cc));
+            }
+          }
           float4 x = *reinterpret_cast<const float4*>(T + r * kTP + cc);
           if (m < p.M) {
             if (EPI == 0 || EPI == 1 || EPI == 4) { x.x += bq.x; x.y += bq.y; x.z += bq.z; x.w += bq.w; }
@@ -305,6 +314,11 @@ __global__ void __launch_bounds__(64 + 32 * epi_warps<EPI>(), 1) k_gemm_bf16(con
               continue;
             }
             if (EPI == 2) { x.x += g[j].x; x.y += g[j].y; x.z += g[j].z; x.w += g[j].w; }
+            if (EPI == 7) {
+              const float4 g = g7[j % 4], z = z7[j % 4];
+              x = make_float4((x.x + g.x) * dsilu_f(z.x), (x.y + g.y) * dsilu_f(z.y), (x.z + g.z) * dsilu_f(z.z),
+                              (x.w + g.w) * dsilu_f(z.w));
+            }
             if (EPI == 3) {
               x.x *= dsilu_fast(g[j].x); x.y *= dsilu_fast(g[j].y); x.z *= dsilu_fast(g[j].z); x.w *= dsilu_fast(g[j].w);
             }
@@ -408,7 +422,8 @@ int gemm_bf16(cudaStream_t st, int64_t M, int N, int K, const bf16* A, int64_t l
   if (p.outh && (reinterpret_cast<uintptr_t>(outh) & 7)) return -1;
   p.auxh = EPI == 6 ? auxh : nullptr;
   if (EPI == 6 && (!auxh || ldaux % 4 || (reinterpret_cast<uintptr_t>(auxh) & 7))) return -1;
-  if ((EPI == 2 || EPI == 3) && !aux) return -1;
+  if ((EPI == 2 || EPI == 3 || EPI == 7) && !aux) return -1;
+  if (EPI == 7 && (!aux2 || (reinterpret_cast<uintptr_t>(aux2) & 15))) return -1;
   p.b_box_rows = N % 64 == 0 ? 64 : 32;
   p.n_chunk = N <= 256 ? N : N / 2;
   if (p.n_chunk > 256 || p.n_chunk % 16) return -1;
@@ -429,7 +444,7 @@ int gemm_bf16(cudaStream_t st, int64_t M, int N, int K, const bf16* A, int64_t l
   size_t smem = 1024 + b_bytes + (size_t)p.a_stages * kATileBytes + t_bytes + 256;
   // a CTA holding more than half of TMEM runs alone on its SM, so allocation never waits
   if (p.tmem_cols > 256 && smem < 120 * 1024) smem = 120 * 1024;
-  static bool attr_set[7] = {false, false, false, false, false, false, false};
+  static bool attr_set[8] = {};
   if (!attr_set[EPI]) {
     cudaFuncSetAttribute(k_gemm_bf16<EPI>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
     attr_set[EPI] = true;
@@ -459,6 +474,9 @@ template int gemm_bf16<4>(cudaStream_t, int64_t, int, int, const bf16*, int64_t,
                           const float*, int, float*, int, bf16*, int, int*, __half*, const float*,
                           const __half*);
 template int gemm_bf16<5>(cudaStream_t, int64_t, int, int, const bf16*, int64_t, const bf16*, const float*,
+                          const float*, int, float*, int, bf16*, int, int*, __half*, const float*,
+                          const __half*);
+template int gemm_bf16<7>(cudaStream_t, int64_t, int, int, const bf16*, int64_t, const bf16*, const float*,
                           const float*, int, float*, int, bf16*, int, int*, __half*, const float*,
                           const __half*);
 template int gemm_bf16<6>(cudaStream_t, int64_t, int, int, const bf16*, int64_t, const bf16*, const float*,

@@ -32,7 +32,7 @@ namespace ctd {
 // (64 x 128, or 128 x 64 / 256 x 32 for narrow outputs), 256 threads, each 8 rows x 4 columns,
 // K staged 32 at a time (A transposed in smem).  Every output is the same fmaf chain over k in
 // increasing order whatever the tile, so the tile shapes give bit-identical results.
-enum Epi { EPI_BIAS = 0, EPI_BIAS_SILU = 1, EPI_ADD = 2, EPI_DSILU = 3 };
+enum Epi { EPI_BIAS = 0, EPI_BIAS_SILU = 1, EPI_ADD = 2, EPI_DSILU = 3, EPI_ADD_DSILU = 4 };
 constexpr int GBM = 64, GBN = 128, GBK = 32;
 
 // Four outputs of row m, columns nb .. nb + 3, with the fused epilogue.
@@ -44,7 +44,8 @@ __device__ __forceinline__ void gemm_store(const float (&acc)[4], int64_t m, int
   for (int j = 0; j < 4; ++j) {
     float x = acc[j];
     if (EPI == EPI_BIAS || EPI == EPI_BIAS_SILU) x += bias ? bias[nb + j] : 0.0f;
-    if (EPI == EPI_ADD) x += aux[m * ldaux + nb + j];
+    if (EPI == EPI_ADD || EPI == EPI_ADD_DSILU) x += aux[m * ldaux + nb + j];
+    if (EPI == EPI_ADD_DSILU) x *= dsilu_f(out2[m * ldo2 + nb + j]);   // out2: the SiLU argument
     if (EPI == EPI_DSILU) x *= dsilu_f(aux[m * ldaux + nb + j]);
     r[j] = x;
   }
@@ -266,6 +267,7 @@ void gemm_f32(cudaStream_t st, int epi, int64_t M, int N, int K, const float* A,
     case EPI_BIAS: gemm<EPI_BIAS>(st, M, N, K, A, lda, B, bias, aux, ldaux, out, ldo, out2, ldo2); break;
     case EPI_BIAS_SILU: gemm<EPI_BIAS_SILU>(st, M, N, K, A, lda, B, bias, aux, ldaux, out, ldo, out2, ldo2); break;
     case EPI_ADD: gemm<EPI_ADD>(st, M, N, K, A, lda, B, bias, aux, ldaux, out, ldo, out2, ldo2); break;
+    case EPI_ADD_DSILU: gemm<EPI_ADD_DSILU>(st, M, N, K, A, lda, B, bias, aux, ldaux, out, ldo, out2, ldo2); break;
     default: gemm<EPI_DSILU>(st, M, N, K, A, lda, B, bias, aux, ldaux, out, ldo, out2, ldo2); break;
   }
 }
