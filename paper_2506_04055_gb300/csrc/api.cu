@@ -245,20 +245,14 @@ int copy_in(ctd_ctx* c, void* dst, const void* src, size_t bytes, bool device) {
   return CTD_OK;
 }
 
-// Per-step prune of the Verlet list to the active list (positions already in c->x_s, sorted).
-int prune(ctd_ctx* c, double* maxdisp_out) {
+// Per-step prune of the Verlet list to the active list (positions already in c->x_s, sorted), in two
+// parts: the displacements since the build (and, if asked for, the largest read back) ...
+int prune_begin(ctd_ctx* c, double* maxdisp_out) {
   StageGuard sg(STG_PRUNE);
   cudaStream_t st = c->st;
-  const int64_t n = c->n, n1 = n > 0 ? n : 1, e1 = c->n_verlet > 0 ? c->n_verlet : 1;
+  const int64_t n = c->n, n1 = n > 0 ? n : 1;
   ENSURE(c, c->delta, sizeof(float4) * n1);
   ENSURE(c, c->maxd, sizeof(unsigned int) * 4);
-  ENSURE(c, c->acount, sizeof(int32_t) * n1);
-  ENSURE(c, c->arow, sizeof(int32_t) * (n1 + 1));
-  ENSURE(c, c->acol, sizeof(int32_t) * e1);
-  ENSURE(c, c->ar, sizeof(float4) * e1);
-  ENSURE(c, c->vidx, sizeof(int32_t) * e1);
-  ENSURE(c, c->arev, sizeof(int32_t) * e1);
-  ENSURE(c, c->aend, sizeof(int32_t) * e1);
   CUDA_OK(c, cudaMemsetAsync(c->maxd.p, 0, sizeof(unsigned int), st));
   launch_delta(st, n, P<double>(c->x_s), P<double>(c->xref_s), P<float4>(c->delta), P<unsigned int>(c->maxd));
   if (maxdisp_out) {
@@ -269,6 +263,21 @@ int prune(ctd_ctx* c, double* maxdisp_out) {
     memcpy(&d2, &bits, sizeof(d2));
     *maxdisp_out = std::sqrt((double)d2);
   }
+  return CTD_OK;
+}
+
+// ... and the active list itself.
+int prune_finish(ctd_ctx* c) {
+  StageGuard sg(STG_PRUNE);
+  cudaStream_t st = c->st;
+  const int64_t n = c->n, n1 = n > 0 ? n : 1, e1 = c->n_verlet > 0 ? c->n_verlet : 1;
+  ENSURE(c, c->acount, sizeof(int32_t) * n1);
+  ENSURE(c, c->arow, sizeof(int32_t) * (n1 + 1));
+  ENSURE(c, c->acol, sizeof(int32_t) * e1);
+  ENSURE(c, c->ar, sizeof(float4) * e1);
+  ENSURE(c, c->vidx, sizeof(int32_t) * e1);
+  ENSURE(c, c->arev, sizeof(int32_t) * e1);
+  ENSURE(c, c->aend, sizeof(int32_t) * e1);
   const float rc2 = (float)(c->desc.rc * c->desc.rc);
   const uint8_t* near = c->use_near ? P<uint8_t>(c->near) : nullptr;
   launch_prune(st, false, n, P<int32_t>(c->vrow), P<int32_t>(c->vcol), P<float4>(c->vbase), P<float4>(c->delta),
@@ -281,6 +290,11 @@ int prune(ctd_ctx* c, double* maxdisp_out) {
                    P<int32_t>(c->arev), P<int32_t>(c->aend));
   CUDA_OK(c, cudaGetLastError());
   return CTD_OK;
+}
+
+int prune(ctd_ctx* c, double* maxdisp_out) {
+  const int r = prune_begin(c, maxdisp_out);
+  return r ? r : prune_finish(c);
 }
 
 // Device bytes per atom of the model's activation buffers (FP32 and, on the BF16 path, the
@@ -415,7 +429,77 @@ int evaluate(ctd_ctx* c, bool need_grad) {
   return CTD_OK;
 }
 
-// positions (device, caller order) are in c->x_user: decide on a rebuild, gather, prune.
+void drop_graph(ctd_ctx* c) {
+  if (c->gexec) cudaGraphExecDestroy(c->gexec);
+  c->gexec = nullptr;
+  c->gkey = c->glast = 0;
+}
+
+// The device work after the rebuild decision: active list, species (gather_z: of a new call; an MD
+// state keeps them sorted) and model.  It has no host decision in it, and below a few ten thousand atoms its
+// seventy launches take the host longer than the device, so it is recorded as a CUDA graph and replayed
+// while everything it bakes in besides device memory contents stays the same: the buffers (by their
+// allocation generation), the atom count, the model options and what is asked for.  The first call of
+// a key runs eagerly (and grows what it needs), the second records; new parameters drop the graph.
+// Larger systems gain nothing (96,000 atoms: the device is never idle) and stay eager, as do the
+// strictly local family (it reads its edge count back), stored filters, models without layers (a memset
+// sized by the Verlet list) and profiled calls (events around each launch).
+int forces_step(ctd_ctx* c, bool need_grad, bool gather_z) {
+  auto body = [&]() -> int {
+    const int r = prune_finish(c);
+    if (r) return r;
+    if (gather_z) launch_gather_i32(c->st, c->n, P<int32_t>(c->perm), P<int32_t>(c->z_user), P<int32_t>(c->z_s));
+    return evaluate(c, need_grad);
+  };
+  auto key_now = [&]() {
+    uint64_t h = 1469598103934665603ull;
+    auto mix = [&](uint64_t v) { h = (h ^ v) * 1099511628211ull; };
+    mix(c->alloc_gen); mix((uint64_t)c->n); mix(need_grad); mix(gather_z);
+    mix(c->mw.tc_adjoint); mix(c->mw.tc_message); mix((uint64_t)c->mw.edge_chunk_rows); mix(c->use_ew); mix(c->use_near);
+    return h == 0 ? 1 : h;
+  };
+  constexpr int64_t kGraphFeatures = (int64_t)1 << 22;   // atoms x width
+  if (c->local() || c->n == 0 || c->desc.T == 0 || c->n * c->desc.F > kGraphFeatures || prof_recording() ||
+      model_stores_edges(c->mw, c->desc.precision))
+    return body();
+  const uint64_t key = key_now();
+  if (!(c->gexec && c->gkey == key) && key == c->glast) {
+    drop_graph(c);
+    cudaGraph_t g = nullptr;
+    int64_t before[STG_COUNT];
+    for (int k = 0; k < STG_COUNT; ++k) before[k] = c->prof.launches[k];
+    c->capturing = true;
+    int r = CTD_ERR_CUDA;
+    if (cudaStreamBeginCapture(c->st, cudaStreamCaptureModeThreadLocal) == cudaSuccess) {
+      r = body();
+      if (cudaStreamEndCapture(c->st, &g) != cudaSuccess) r = CTD_ERR_CUDA;
+    }
+    c->capturing = false;
+    if (r == CTD_OK && g && key_now() == key && cudaGraphInstantiate(&c->gexec, g, 0) == cudaSuccess) {
+      c->gkey = key;
+    } else {
+      c->gexec = nullptr;
+      cudaGetLastError();
+      c->err.clear();
+    }
+    if (g) cudaGraphDestroy(g);
+    for (int k = 0; k < STG_COUNT; ++k) {   // counted when the graph is launched
+      c->glaunches[k] = c->prof.launches[k] - before[k];
+      c->prof.launches[k] = before[k];
+    }
+  }
+  if (c->gexec && c->gkey == key) {
+    CUDA_OK(c, cudaGraphLaunch(c->gexec, c->st));
+    for (int k = 0; k < STG_COUNT; ++k) c->prof.launches[k] += c->glaunches[k];
+    return CTD_OK;
+  }
+  const bool tried = c->glast == key;   // the capture did not complete: not again for this key
+  const int r = body();
+  c->glast = r == CTD_OK && !tried ? key_now() : 0;
+  return r;
+}
+
+// positions (device, caller order) are in c->x_user: decide on a rebuild, gather, displacements.
 int prepare_step(ctd_ctx* c, int64_t n, const double H[9], bool force_rebuild, int32_t* rebuilt, double* maxdisp) {
   bool need = force_rebuild || !c->have_list || n != c->n || memcmp(H, c->H, sizeof(double) * 9) != 0 ||
               c->cutoff < c->desc.rc;
@@ -423,7 +507,7 @@ int prepare_step(ctd_ctx* c, int64_t n, const double H[9], bool force_rebuild, i
   if (!need) {
     launch_gather_positions(c->st, n, P<int32_t>(c->perm), P<double>(c->x_user), P<double>(c->x_s));
     double md = 0.0;
-    int r = prune(c, &md);
+    int r = prune_begin(c, &md);
     if (r) return r;
     const double eff_skin = c->cutoff + c->skin - c->desc.rc;
     if (md > 0.5 * eff_skin || !std::isfinite(md)) need = true;
@@ -436,7 +520,7 @@ int prepare_step(ctd_ctx* c, int64_t n, const double H[9], bool force_rebuild, i
     *rebuilt = 1;
     launch_gather_positions(c->st, n, P<int32_t>(c->perm), P<double>(c->x_user), P<double>(c->x_s));
     double md = 0.0;
-    r = prune(c, &md);
+    r = prune_begin(c, &md);
     if (r) return r;
     *maxdisp = md;
   }
@@ -564,6 +648,7 @@ int load_local_params(ctd_ctx* c, const char* b, size_t nbytes) {
 }
 
 int load_params_impl(ctd_ctx* c, const void* blob, size_t nbytes) {
+  drop_graph(c);
   if (!blob || nbytes < 64) return fail(c, CTD_ERR_INVALID_ARG, "parameter blob too short");
   const char* b = static_cast<const char*>(blob);
   if (c->local()) return load_local_params(c, b, nbytes);
@@ -778,6 +863,7 @@ int ctd_create(ctd_ctx** out, const ctd_model_desc* desc, size_t hbm_budget_byte
 void ctd_destroy(ctd_ctx* c) {
   if (!c) return;
   if (c->st) cudaStreamSynchronize(c->st);
+  drop_graph(c);
   c->prof.collect();
   for (DBuf* b : c->all)
     if (b->p) cudaFree(b->p);
@@ -958,11 +1044,17 @@ int ctd_compute(ctd_ctx* c, int64_t n, const int32_t* species, const double* pos
   double md = 0.0;
   r = prepare_step(c, n, cell, flags & CTD_REBUILD, &rebuilt, &md);
   if (r) return r;
-  launch_gather_i32(c->st, n, P<int32_t>(c->perm), P<int32_t>(c->z_user), P<int32_t>(c->z_s));
-  if (timing) cudaEventRecord(ev[1], c->st);
   const bool need_grad = flags & (CTD_NEED_FORCES | CTD_NEED_VIRIAL);
   CUDA_OK(c, cudaMemsetAsync(c->status.p, 0, sizeof(int32_t), c->st));
-  r = evaluate(c, need_grad);
+  if (timing) {   // the active list counts as neighbour time
+    r = prune_finish(c);
+    if (r) return r;
+    launch_gather_i32(c->st, n, P<int32_t>(c->perm), P<int32_t>(c->z_user), P<int32_t>(c->z_s));
+    cudaEventRecord(ev[1], c->st);
+    r = evaluate(c, need_grad);
+  } else {
+    r = forces_step(c, need_grad, true);
+  }
   if (r) return r;
   if (timing) cudaEventRecord(ev[2], c->st);
   // outputs
@@ -1117,17 +1209,17 @@ int md_rebuild(ctd_ctx* c) {
 
 int md_forces(ctd_ctx* c, int32_t* rebuilds) {
   double md = 0.0;
-  int r = prune(c, &md);
+  int r = prune_begin(c, &md);
   if (r) return r;
   if (md > 0.5 * c->skin || !std::isfinite(md)) {
     if (!std::isfinite(md)) return fail(c, CTD_ERR_NONFINITE, "non-finite positions in MD");
     r = md_rebuild(c);
     if (r) return r;
     ++*rebuilds;
-    r = prune(c, nullptr);
+    r = prune_begin(c, nullptr);
     if (r) return r;
   }
-  return evaluate(c, true);
+  return forces_step(c, true, false);
 }
 }  // namespace
 

@@ -39,6 +39,11 @@ struct ctd_ctx {
   bool capturing = false;
   uint64_t alloc_gen = 0;
   std::vector<DBuf*> all;
+  // recorded forces step of a call or MD step (api.cu, forces_step): its key, the key of the last
+  // eager step, and the launches it holds per stage
+  cudaGraphExec_t gexec = nullptr;
+  uint64_t gkey = 0, glast = 0;
+  int64_t glaunches[ctd::STG_COUNT] = {};
 
   // parameters
   bool have_params = false;
@@ -113,6 +118,7 @@ int setup_geometry_into(ctd_ctx* c, CellGeom& g, int64_t* ncell, const double H[
 int check_status(ctd_ctx* c);
 int copy_in(ctd_ctx* c, void* dst, const void* src, size_t bytes, bool device);
 int prune(ctd_ctx* c, double* maxdisp_out);
+void drop_graph(ctd_ctx* c);
 int evaluate(ctd_ctx* c, bool need_grad);
 size_t model_bytes_per_atom(const ctd_ctx* c);
 
