@@ -353,8 +353,10 @@ int evaluate_local(ctd_ctx* c, bool need_grad) {
     launch_forces(st, n, P<int32_t>(c->arow), P<float4>(c->ar), P<int32_t>(c->arev), P<float4>(c->hedge),
                   P<float>(c->force_s), P<double>(c->vpart), kPartials, P<int>(c->status));
   }
-  launch_sum_partials(st, kPartials, 1, P<double>(c->epart), P<double>(c->out_e), 1.0);
-  if (need_grad) launch_sum_partials(st, kPartials, 9, P<double>(c->vpart), P<double>(c->out_w), 1.0);
+  if (need_grad)
+    launch_sum_energy_virial(st, kPartials, P<double>(c->epart), P<double>(c->vpart), P<double>(c->out_e), P<double>(c->out_w));
+  else
+    launch_sum_partials(st, kPartials, 1, P<double>(c->epart), P<double>(c->out_e), 1.0);
   CUDA_OK(c, cudaGetLastError());
   return CTD_OK;
 }
@@ -423,8 +425,10 @@ int evaluate(ctd_ctx* c, bool need_grad) {
                                 kPartials, P<float>(c->eatom), P<int>(c->status), wst, wlayer, ew);
   }
   StageGuard sg(STG_FORCES);
-  launch_sum_partials(st, kPartials, 1, P<double>(c->epart), P<double>(c->out_e), 1.0);
-  if (need_grad) launch_sum_partials(st, kPartials, 9, P<double>(c->vpart), P<double>(c->out_w), 1.0);
+  if (need_grad)
+    launch_sum_energy_virial(st, kPartials, P<double>(c->epart), P<double>(c->vpart), P<double>(c->out_e), P<double>(c->out_w));
+  else
+    launch_sum_partials(st, kPartials, 1, P<double>(c->epart), P<double>(c->out_e), 1.0);
   CUDA_OK(c, cudaGetLastError());
   return CTD_OK;
 }

@@ -150,10 +150,10 @@ __global__ void k_kinetic(int64_t n, const double* __restrict__ mass, const doub
 // result is deterministic.  (A single warp walking the partials one by one spent ~170 us on
 // GB300's FP64 latency chain for 608 partials.)
 constexpr int kSumThreads = 256;
-__global__ void __launch_bounds__(kSumThreads) k_sum_partials(int nb, int width, const double* __restrict__ partials,
-                                                              double* __restrict__ out, double scale) {
+__device__ __forceinline__ void sum_column(int nb, int width, int c, const double* __restrict__ partials, double* out,
+                                           double scale) {
   __shared__ double ss[kSumThreads], sc[kSumThreads];
-  const int c = blockIdx.x, tid = threadIdx.x;
+  const int tid = threadIdx.x;
   double s = 0.0, comp = 0.0;
   for (int b = tid; b < nb; b += kSumThreads) {
     const double x = partials[(int64_t)b * width + c], t = s + x;
@@ -172,7 +172,18 @@ __global__ void __launch_bounds__(kSumThreads) k_sum_partials(int nb, int width,
     }
     __syncthreads();
   }
-  if (tid == 0) out[c] = (ss[0] + sc[0]) * scale;
+  if (tid == 0) *out = (ss[0] + sc[0]) * scale;
+}
+__global__ void __launch_bounds__(kSumThreads) k_sum_partials(int nb, int width, const double* __restrict__ partials,
+                                                              double* __restrict__ out, double scale) {
+  sum_column(nb, width, blockIdx.x, partials, out + blockIdx.x, scale);
+}
+// The energy (block 0) and the nine virial components of a call in one launch.
+__global__ void __launch_bounds__(kSumThreads) k_sum_energy_virial(int nb, const double* __restrict__ epart,
+                                                                   const double* __restrict__ vpart, double* __restrict__ e,
+                                                                   double* __restrict__ w) {
+  if (blockIdx.x == 0) sum_column(nb, 1, 0, epart, e, 1.0);
+  else sum_column(nb, 9, blockIdx.x - 1, vpart, w + blockIdx.x - 1, 1.0);
 }
 
 // out[perm[k]] = (double) in[k]  for [n][w] rows
@@ -256,6 +267,10 @@ void launch_kinetic(cudaStream_t st, int64_t n, const double* m, const double* v
 void launch_sum_partials(cudaStream_t st, int nb, int width, const double* partials, double* out, double scale) {
   if (width < 1) return;
   { LaunchScope ls_(st); k_sum_partials<<<width, kSumThreads, 0, st>>>(nb, width, partials, out, scale); }
+}
+void launch_sum_energy_virial(cudaStream_t st, int nb, const double* epart, const double* vpart, double* e, double* w) {
+  LaunchScope ls_(st);
+  k_sum_energy_virial<<<10, kSumThreads, 0, st>>>(nb, epart, vpart, e, w);
 }
 void launch_scatter_rows(cudaStream_t st, int64_t n, int w, const int32_t* perm, const float* in, double* out) {
   if (n) { LaunchScope ls_(st); k_scatter_rows<<<nblk(n * w), kThreads, 0, st>>>(n, w, perm, in, out); }
