@@ -218,13 +218,14 @@ __global__ __launch_bounds__((BM / TM) * (BN / 4)) void k_gemm_small(
   }
 }
 
-constexpr int kMidK = 512, kSmallK = 768;   // largest K of the two tile shapes (3F = 768 at F = 256)
+// largest K of the tile shapes (3F = 768 at F = 256): 8 TM x 64 tiles up to TM = 4, above it, 16 x 32 tiles
+constexpr int kMidK = 512, kTallK = 384, kSmallK = 768;
 template <int EPI, int BM, int BN, int TM>
 static void launch_gemm_small(cudaStream_t st, int64_t M, int N, int K, const float* A, int lda, const float* B,
                               const float* bias, const float* aux, int ldaux, float* out, int ldo, float* out2, int ldo2) {
   static const cudaError_t attr = cudaFuncSetAttribute(
       k_gemm_small<EPI, BM, BN, TM>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-      (int)gemm_small_smem<BM, BN>(BM == 32 ? kMidK : kSmallK));
+      (int)gemm_small_smem<BM, BN>(BN == 32 ? kSmallK : TM <= 4 ? kMidK : kTallK));
   (void)attr;
   const unsigned grid = (unsigned)(((M + BM - 1) / BM) * ((N + BN - 1) / BN));
   LaunchScope ls_(st);
@@ -239,12 +240,27 @@ static void gemm_tiled(cudaStream_t st, int64_t M, int N, int K, const float* A,
   constexpr int BM = 8 * (256 / (BN / 4));
   const int64_t tiles = (int64_t)((N + BN - 1) / BN) * ((M + BM - 1) / BM);
   if (tiles < 2 * 152 && K <= kSmallK) {   // under two waves of the 256-thread tiles
-    const int64_t mid = ((M + 31) / 32) * ((N + 63) / 64);
-    // 32 x 64 tiles once they fill the SMs, 16 x 32 tiles below that
-    if (mid >= 152 && K <= kMidK)
-      launch_gemm_small<EPI, 32, 64, 4>(st, M, N, K, A, lda, B, bias, aux, ldaux, out, ldo, out2, ldo2);
-    else
+    const int64_t cols = (N + 63) / 64, mid = ((M + 31) / 32) * cols;
+    // 8 TM x 64 tiles once 32 rows of them fill the SMs, 16 x 32 tiles below that.  All tiles of an
+    // SM run together, so a launch takes as long as the SM with the most: TM is the height whose
+    // tiles per SM, times their work, is least (1.5 rows for what does not grow with TM): 5,997 atoms,
+    // N = 64: 188 tiles of 32 rows put two on some SMs, 150 of 40 rows one on each (the GEMMs of a
+    // call 251 us, now 234)
+    if (mid >= 152 && K <= kMidK) {
+      int tm = 4;
+      double least = 0.0;
+      for (int t = 3; t <= (K <= kTallK ? 6 : 4); ++t) {
+        const int64_t per_sm = (((M + 8 * t - 1) / (8 * t)) * cols + 151) / 152;
+        if (t > 4 && K > 128 && per_sm > 2) continue;   // fewer than three of them fit an SM's shared memory
+        const double work = (double)per_sm * (t + 1.5);
+        if (least == 0.0 || work < least) { least = work; tm = t; }
+      }
+      auto go = tm == 3 ? launch_gemm_small<EPI, 24, 64, 3> : tm == 4 ? launch_gemm_small<EPI, 32, 64, 4>
+              : tm == 5 ? launch_gemm_small<EPI, 40, 64, 5> : launch_gemm_small<EPI, 48, 64, 6>;
+      go(st, M, N, K, A, lda, B, bias, aux, ldaux, out, ldo, out2, ldo2);
+    } else {
       launch_gemm_small<EPI, 16, 32, 1>(st, M, N, K, A, lda, B, bias, aux, ldaux, out, ldo, out2, ldo2);
+    }
     return;
   }
   LaunchScope ls_(st);
