@@ -38,6 +38,7 @@ struct GemmBf16Args {
   __half* outh;   // EPI 0, 1 and 4: FP16 copy of out, same element stride ldo (optional; EPI 1: the
                   // SiLU argument; EPI 4: the message table)
   int* status;
+  int nsplit;   // CTAs that share a row tile, N / nsplit columns each
   int a_stages, n_acc, b_box_rows, n_chunk;   // a_stages: k-block stages of the A ring
   uint32_t tmem_cols;
 };
@@ -65,7 +66,8 @@ __global__ void __launch_bounds__(64 + 32 * epi_warps<EPI>(), 1) k_gemm_bf16(con
   unsigned char* smem = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
   constexpr int kEpiWarps = epi_warps<EPI>(), kEpiGroups = kEpiWarps / 4;
   const int KB = (p.K + kBlockK - 1) / kBlockK;   // a ragged last block is zero-filled by the TMA
-  const int N = p.N;
+  const int N = p.N / p.nsplit, n0 = (int)(blockIdx.x % p.nsplit) * N;   // this CTA's columns n0 .. n0 + N - 1
+  const int64_t tile0 = blockIdx.x / p.nsplit, tile_step = gridDim.x / p.nsplit;
   unsigned char* sB = smem;                                        // KB x N x 128 B
   unsigned char* sA = sB + (size_t)KB * N * 128;                   // a_stages x 16 KB
   float* sT = reinterpret_cast<float*>(sA + (size_t)p.a_stages * kATileBytes);   // kEpiWarps x 32 x kTP
@@ -108,9 +110,9 @@ __global__ void __launch_bounds__(64 + 32 * epi_warps<EPI>(), 1) k_gemm_bf16(con
       umma::mbar_expect_tx(bbar, (uint32_t)(N * KB * kBlockK * 2));   // whole boxes, fill included
       for (int kb = 0; kb < KB; ++kb)
         for (int r0 = 0; r0 < N; r0 += p.b_box_rows)
-          umma::tma_load_2d(sB + (size_t)kb * N * 128 + (size_t)r0 * 128, &tmB, kb * kBlockK, r0, bbar);
+          umma::tma_load_2d(sB + (size_t)kb * N * 128 + (size_t)r0 * 128, &tmB, kb * kBlockK, n0 + r0, bbar);
       int64_t g = 0;   // k-blocks loaded so far
-      for (int64_t tile = blockIdx.x; ok && tile < ntiles; tile += gridDim.x) {
+      for (int64_t tile = tile0; ok && tile < ntiles; tile += tile_step) {
         for (int kb = 0; kb < KB; ++kb, ++g) {
           const int s = (int)(g % p.a_stages);
           const int64_t u = g / p.a_stages;
@@ -126,7 +128,7 @@ __global__ void __launch_bounds__(64 + 32 * epi_warps<EPI>(), 1) k_gemm_bf16(con
       int it = 0;
       int64_t g = 0;   // k-blocks consumed so far
       const uint32_t idesc = umma::idesc_bf16_m128(p.n_chunk);
-      for (int64_t tile = blockIdx.x; ok && tile < ntiles; tile += gridDim.x, ++it) {
+      for (int64_t tile = tile0; ok && tile < ntiles; tile += tile_step, ++it) {
         const int a = it % p.n_acc;
         if (it >= p.n_acc && !umma::mbar_wait(&tempty[a], ((it / p.n_acc) - 1) & 1)) { ok = false; break; }
         for (int kb = 0; kb < KB; ++kb, ++g) {
@@ -171,7 +173,7 @@ __global__ void __launch_bounds__(64 + 32 * epi_warps<EPI>(), 1) k_gemm_bf16(con
       return umma::mbar_wait(&gbar[grp], (gph++) & 1);
     };
     int it = 0;
-    for (int64_t tile = blockIdx.x; ok && tile < ntiles; tile += gridDim.x, ++it) {
+    for (int64_t tile = tile0; ok && tile < ntiles; tile += tile_step, ++it) {
       const int a = it % p.n_acc;
       if (!umma::mbar_wait(&tfull[a], (it / p.n_acc) & 1)) { ok = false; break; }
       umma::fence_after();
@@ -182,9 +184,9 @@ __global__ void __launch_bounds__(64 + 32 * epi_warps<EPI>(), 1) k_gemm_bf16(con
         if (lane == 0) umma::mbar_arrive(&tempty[a]);
       }
       for (int ch = grp; ch < nchunks; ch += kEpiGroups) {
-        const int c0 = 32 * ch;
+        const int c0 = n0 + 32 * ch;   // first output column of the chunk
         float v[32];
-        umma::tmem_ld32(tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(a * N + c0), v);
+        umma::tmem_ld32(tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(a * N + 32 * ch), v);
         if (ch + kEpiGroups >= nchunks) {
           // the accumulator has been read: the MMA of a later tile may reuse it
           umma::fence_before();
@@ -200,7 +202,7 @@ __global__ void __launch_bounds__(64 + 32 * epi_warps<EPI>(), 1) k_gemm_bf16(con
         if ((EPI == 0 || EPI == 1 || EPI == 4) && p.bias) bq = *reinterpret_cast<const float4*>(p.bias + c0 + cc);
         // EPI 4 (phi packing, N = 3F): columns [phi_s | phi_vv | phi_vs]; row m of PHI (6F) gets
         // [phi_s | v_0 phi_vv | v_1 phi_vv | v_2 phi_vv | phi_vs | phi_vv], v from aux ([n][3F])
-        const int Fb = N / 3, blk = EPI == 4 ? c0 / Fb : 0, f0 = c0 - blk * Fb + cc;
+        const int Fb = p.N / 3, blk = EPI == 4 ? c0 / Fb : 0, f0 = c0 - blk * Fb + cc;
         float4 gv[EPI == 4 ? 8 : 1][3];
         if (EPI == 4 && blk == 1) {
           // aux null: v = 0 (first layer), psi = 0
@@ -235,8 +237,8 @@ __global__ void __launch_bounds__(64 + 32 * epi_warps<EPI>(), 1) k_gemm_bf16(con
               const float4 gk = __ldg(reinterpret_cast<const float4*>(p.aux + (3 * ai + k) * p.ldaux + c0 + fq));
               x[k] = make_float4(t.x + gk.x, t.y + gk.y, t.z + gk.z, t.w + gk.w);
             }
-            const float4 gs = __ldg(reinterpret_cast<const float4*>(p.aux2 + ai * N + c0 + fq));
-            float4* o = reinterpret_cast<float4*>(p.out + (ai * N + c0 + fq) * 4);
+            const float4 gs = __ldg(reinterpret_cast<const float4*>(p.aux2 + ai * p.N + c0 + fq));
+            float4* o = reinterpret_cast<float4*>(p.out + (ai * p.N + c0 + fq) * 4);
             o[0] = make_float4(gs.x, x[0].x, x[1].x, x[2].x);
             o[1] = make_float4(gs.y, x[0].y, x[1].y, x[2].y);
             o[2] = make_float4(gs.z, x[0].z, x[1].z, x[2].z);
@@ -271,7 +273,7 @@ __global__ void __launch_bounds__(64 + 32 * epi_warps<EPI>(), 1) k_gemm_bf16(con
             for (int q = 0; q < 4; ++q) {
               const int64_t mq = m + 4 * q < p.M ? m + 4 * q : p.M - 1;
               g7[q] = __ldg(reinterpret_cast<const float4*>(p.aux + mq * p.ldaux + c0 + cc));
-              z7[q] = __ldg(reinterpret_cast<const float4*>(p.aux2 + mq * N + c0 + cc));
+              z7[q] = __ldg(reinterpret_cast<const float4*>(p.aux2 + mq * p.N + c0 + cc));
             }
           }
           float4 x = *reinterpret_cast<const float4*>(T + r * kTP + cc);
@@ -424,20 +426,28 @@ int gemm_bf16(cudaStream_t st, int64_t M, int N, int K, const bf16* A, int64_t l
   if (EPI == 6 && (!auxh || ldaux % 4 || (reinterpret_cast<uintptr_t>(auxh) & 7))) return -1;
   if ((EPI == 2 || EPI == 3 || EPI == 7) && !aux) return -1;
   if (EPI == 7 && (!aux2 || (reinterpret_cast<uintptr_t>(aux2) & 15))) return -1;
-  p.b_box_rows = N % 64 == 0 ? 64 : 32;
-  p.n_chunk = N <= 256 ? N : N / 2;
+  // Few row tiles: each is shared by as many CTAs as keep the grid within the SMs, down to 32 columns
+  // each (every output element is the same accumulation).  One CTA per tile left a launch over 500
+  // rows to four SMs, each loading all of W and storing up to 384 columns (8 to 18 us).
+  const int64_t ntiles = (M + tile_rows<EPI>() - 1) / tile_rows<EPI>();
+  p.nsplit = 1;
+  for (int s = 2; s <= N / 32; ++s)
+    if ((N / 32) % s == 0 && ntiles * s <= num_sms()) p.nsplit = s;
+  const int Nc = N / p.nsplit;   // columns of a CTA
+  p.b_box_rows = Nc % 64 == 0 ? 64 : 32;
+  p.n_chunk = Nc <= 256 ? Nc : Nc / 2;
   if (p.n_chunk > 256 || p.n_chunk % 16) return -1;
   const int KB = (K + kBlockK - 1) / kBlockK;
-  const size_t b_bytes = (size_t)KB * N * 128;
+  const size_t b_bytes = (size_t)KB * Nc * 128;
   constexpr int kEpiWarps = epi_warps<EPI>();
   const size_t t_bytes = (size_t)kEpiWarps * 32 * kTP * sizeof(float);
   const size_t limit = 227 * 1024 - 1024 - 256 - t_bytes;
   if (b_bytes + 2 * (size_t)kATileBytes > limit) return -1;
   p.a_stages = (int)((limit - b_bytes) / kATileBytes);
   if (p.a_stages > kMaxAStages) p.a_stages = kMaxAStages;
-  p.n_acc = 2 * N <= 512 ? 2 : 1;
+  p.n_acc = 2 * Nc <= 512 ? 2 : 1;
   uint32_t cols = 32;
-  while (cols < (uint32_t)(p.n_acc * N)) cols <<= 1;
+  while (cols < (uint32_t)(p.n_acc * Nc)) cols <<= 1;
   p.tmem_cols = cols;
   CUtensorMap ta, tb;
   if (!make_tmap_bf16(&ta, A, M, K, lda, kTileM) || !make_tmap_bf16(&tb, W, N, K, K, p.b_box_rows)) return -2;
@@ -449,8 +459,7 @@ int gemm_bf16(cudaStream_t st, int64_t M, int N, int K, const bf16* A, int64_t l
     cudaFuncSetAttribute(k_gemm_bf16<EPI>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
     attr_set[EPI] = true;
   }
-  const int64_t ntiles = (M + tile_rows<EPI>() - 1) / tile_rows<EPI>();
-  const int grid = (int)(ntiles < num_sms() ? ntiles : num_sms());
+  const int grid = (int)(ntiles * p.nsplit < num_sms() ? ntiles * p.nsplit : num_sms());
   {
     LaunchScope ls_(st);
     k_gemm_bf16<EPI><<<grid, 64 + 32 * kEpiWarps, smem, st>>>(ta, tb, p);
