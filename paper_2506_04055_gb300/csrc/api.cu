@@ -319,11 +319,17 @@ size_t model_bytes_per_atom(const ctd_ctx* c) {
   return bytes;
 }
 
+// Blocks of the energy, virial and kinetic partial sums: one per eight atoms (a warp each in the force
+// kernel) up to kPartials.  Each block ends in a few FP64 operations, at a sixty-fourth of the FP32 rate: 608 blocks
+// over 192 atoms spent half of the force kernel's 12 us there.
+int partials_for(int64_t n) { return (int)std::min<int64_t>(kPartials, std::max<int64_t>(1, (n + 7) / 8)); }
+
 // Model evaluation on the current active list; forces (sorted, FP32) in c->force_s,
 // energy in c->out_e[0], virial in c->out_w[0..8], per-atom energies (sorted) in c->eatom.
 // The strictly local model: edge arrays sized by this step's active edge count.
 int evaluate_local(ctd_ctx* c, bool need_grad) {
   cudaStream_t st = c->st;
+  const int np = partials_for(c->n);
   const int64_t n = c->n, n1 = n > 0 ? n : 1, e1 = c->n_verlet > 0 ? c->n_verlet : 1;
   int32_t act = 0;
   if (n > 0) {
@@ -344,19 +350,19 @@ int evaluate_local(ctd_ctx* c, bool need_grad) {
   ENSURE(c, c->status, sizeof(int32_t) * 4);
   const int bad = local_forward_backward(st, c->lw, n, E, P<int32_t>(c->z_s), P<int32_t>(c->arow),
                                          P<int32_t>(c->acol), P<float4>(c->ar), P<float>(c->lbuf), need_grad, ew,
-                                         P<double>(c->epart), kPartials, P<float>(c->eatom), P<float4>(c->hedge),
+                                         P<double>(c->epart), np, P<float>(c->eatom), P<float4>(c->hedge),
                                          P<int>(c->status));
   if (bad) return fail(c, CTD_ERR_INVALID_ARG, "local model, BF16 path: unsupported GEMM shape");
   StageGuard sg(STG_FORCES);
   if (need_grad) {
     if (E == 0) CUDA_OK(c, cudaMemsetAsync(c->hedge.p, 0, sizeof(float4), st));
     launch_forces(st, n, P<int32_t>(c->arow), P<float4>(c->ar), P<int32_t>(c->arev), P<float4>(c->hedge),
-                  P<float>(c->force_s), P<double>(c->vpart), kPartials, P<int>(c->status));
+                  P<float>(c->force_s), P<double>(c->vpart), np, P<int>(c->status));
   }
   if (need_grad)
-    launch_sum_energy_virial(st, kPartials, P<double>(c->epart), P<double>(c->vpart), P<double>(c->out_e), P<double>(c->out_w));
+    launch_sum_energy_virial(st, np, P<double>(c->epart), P<double>(c->vpart), P<double>(c->out_e), P<double>(c->out_w));
   else
-    launch_sum_partials(st, kPartials, 1, P<double>(c->epart), P<double>(c->out_e), 1.0);
+    launch_sum_partials(st, np, 1, P<double>(c->epart), P<double>(c->out_e), 1.0);
   CUDA_OK(c, cudaGetLastError());
   return CTD_OK;
 }
@@ -365,7 +371,7 @@ int evaluate(ctd_ctx* c, bool need_grad) {
   if (c->local()) return evaluate_local(c, need_grad);
   cudaStream_t st = c->st;
   const int64_t n = c->n, n1 = n > 0 ? n : 1, e1 = c->n_verlet > 0 ? c->n_verlet : 1;
-  const int F = c->desc.F, T = c->desc.T;
+  const int F = c->desc.F, T = c->desc.T, np = partials_for(c->n);
   const int nb = model_buffer_count();
   if ((int)c->mbuf.size() < nb) c->mbuf.resize(nb);
   std::vector<float*> ptrs(nb, nullptr);
@@ -414,21 +420,21 @@ int evaluate(ctd_ctx* c, bool need_grad) {
     }
     int bad = model_forward_backward_bf16(st, c->mw, n, P<int32_t>(c->z_s), P<int32_t>(c->arow), P<int32_t>(c->acol),
                                           P<float4>(c->ar), P<int32_t>(c->arev), ptrs.data(), bptrs.data(), need_grad,
-                                          P<double>(c->epart), kPartials, P<float4>(c->hedge), P<float>(c->force_s),
-                                          P<double>(c->vpart), kPartials, P<float>(c->eatom), P<int>(c->status),
+                                          P<double>(c->epart), np, P<float4>(c->hedge), P<float>(c->force_s),
+                                          P<double>(c->vpart), np, P<float>(c->eatom), P<int>(c->status),
                                           wst, wlayer, P<int32_t>(c->aend), ew);
     if (bad) return fail(c, CTD_ERR_INVALID_ARG, "BF16 path: unsupported GEMM shape");
   } else {
     model_forward_backward_fp32(st, c->mw, n, P<int32_t>(c->z_s), P<int32_t>(c->arow), P<int32_t>(c->acol),
                                 P<float4>(c->ar), P<int32_t>(c->arev), ptrs.data(), need_grad, P<double>(c->epart),
-                                kPartials, P<float4>(c->hedge), P<float>(c->force_s), P<double>(c->vpart),
-                                kPartials, P<float>(c->eatom), P<int>(c->status), wst, wlayer, ew);
+                                np, P<float4>(c->hedge), P<float>(c->force_s), P<double>(c->vpart),
+                                np, P<float>(c->eatom), P<int>(c->status), wst, wlayer, ew);
   }
   StageGuard sg(STG_FORCES);
   if (need_grad)
-    launch_sum_energy_virial(st, kPartials, P<double>(c->epart), P<double>(c->vpart), P<double>(c->out_e), P<double>(c->out_w));
+    launch_sum_energy_virial(st, np, P<double>(c->epart), P<double>(c->vpart), P<double>(c->out_e), P<double>(c->out_w));
   else
-    launch_sum_partials(st, kPartials, 1, P<double>(c->epart), P<double>(c->out_e), 1.0);
+    launch_sum_partials(st, np, 1, P<double>(c->epart), P<double>(c->out_e), 1.0);
   CUDA_OK(c, cudaGetLastError());
   return CTD_OK;
 }
@@ -1065,11 +1071,9 @@ int ctd_compute(ctd_ctx* c, int64_t n, const int32_t* species, const double* pos
   ENSURE(c, c->out_f, sizeof(double) * 3 * n1);
   ENSURE(c, c->out_eatom, sizeof(double) * n1);
   double* fdst = (flags & CTD_NEED_FORCES) ? (dev ? forces : P<double>(c->out_f)) : nullptr;
-  if (fdst) launch_scatter_rows(c->st, n, 3, P<int32_t>(c->perm), P<float>(c->force_s), fdst);
   double* edst = c->energy_out_user ? (dev ? c->energy_out_user : P<double>(c->out_eatom)) : nullptr;
-  if (edst) launch_scatter_rows(c->st, n, 1, P<int32_t>(c->perm), P<float>(c->eatom), edst);
-  launch_check_finite(c->st, 1, P<double>(c->out_e), P<int>(c->status));
-  if (fdst) launch_check_finite(c->st, 3 * n, fdst, P<int>(c->status));
+  launch_outputs(c->st, n, P<int32_t>(c->perm), P<float>(c->force_s), P<float>(c->eatom), P<double>(c->out_e), fdst, edst,
+                 P<int>(c->status));
   if (dev) {
     CUDA_OK(c, cudaMemcpyAsync(energy, c->out_e.p, sizeof(double), cudaMemcpyDeviceToDevice, c->st));
     if (flags & CTD_NEED_VIRIAL)
@@ -1233,6 +1237,7 @@ int ctd_md_run(ctd_ctx* c, int32_t nsteps, double dt, double* epot, double* ekin
   if (!c->md_ready) return fail(c, CTD_ERR_STATE, "no MD state");
   if (nsteps < 0 || !(dt > 0.0)) return fail(c, CTD_ERR_INVALID_ARG, "bad step count or time step");
   const int64_t n = c->n;
+  const int nkp = partials_for(n);
   cudaStream_t st = c->st;
   ENSURE(c, c->md_ep, sizeof(double) * ((size_t)nsteps + 1));
   ENSURE(c, c->md_ek, sizeof(double) * ((size_t)nsteps + 1));
@@ -1262,8 +1267,8 @@ int ctd_md_run(ctd_ctx* c, int32_t nsteps, double dt, double* epot, double* ekin
   double* gscale = nvt ? P<double>(c->nhc_state) + np.M * 2 : nullptr;
   auto record = [&](int step) {
     cudaMemcpyAsync(P<double>(c->md_ep) + step, c->out_e.p, sizeof(double), cudaMemcpyDeviceToDevice, st);
-    launch_kinetic(st, n, P<double>(c->md_m), P<double>(c->md_v), P<double>(c->kpart), kPartials);
-    launch_sum_partials(st, kPartials, 1, P<double>(c->kpart), P<double>(c->md_ek) + step, 1.0);
+    launch_kinetic(st, n, P<double>(c->md_m), P<double>(c->md_v), P<double>(c->kpart), nkp);
+    launch_sum_partials(st, nkp, 1, P<double>(c->kpart), P<double>(c->md_ek) + step, 1.0);
     if (nvt) launch_nhc_energy(st, np, P<double>(c->nhc_state), P<double>(c->md_eth) + step);
   };
   record(0);
@@ -1275,8 +1280,8 @@ int ctd_md_run(ctd_ctx* c, int32_t nsteps, double dt, double* epot, double* ekin
     if (r) return r;
     launch_kick(st, n, dt, P<float>(c->force_s), P<double>(c->md_m), P<double>(c->md_v));
     if (nvt) {
-      launch_kinetic(st, n, P<double>(c->md_m), P<double>(c->md_v), P<double>(c->kpart), kPartials);
-      launch_sum_partials(st, kPartials, 1, P<double>(c->kpart), P<double>(c->nhc_ke), 1.0);
+      launch_kinetic(st, n, P<double>(c->md_m), P<double>(c->md_v), P<double>(c->kpart), nkp);
+      launch_sum_partials(st, nkp, 1, P<double>(c->kpart), P<double>(c->nhc_ke), 1.0);
       launch_nhc_half(st, np, 0.5 * dt, P<double>(c->nhc_ke), P<double>(c->nhc_state));
       launch_scale_v(st, n, gscale, P<double>(c->md_v));
     }

@@ -224,8 +224,9 @@ void launch_scale_v_rep(cudaStream_t st, int64_t n, const int32_t* rep, const do
 void launch_kick(cudaStream_t st, int64_t n, double dt, const float* f, const double* m, double* v);
 void launch_kinetic(cudaStream_t st, int64_t n, const double* m, const double* v, double* partials, int nb);
 void launch_sum_partials(cudaStream_t st, int nb, int width, const double* partials, double* out, double scale);
+void launch_outputs(cudaStream_t st, int64_t n, const int32_t* perm, const float* force_s, const float* eatom,
+                    const double* energy, double* force, double* energies, int* status);
 void launch_sum_energy_virial(cudaStream_t st, int nb, const double* epart, const double* vpart, double* e, double* w);
-void launch_scatter_rows(cudaStream_t st, int64_t n, int w, const int32_t* perm, const float* in, double* out);
 void launch_scatter_rows_d(cudaStream_t st, int64_t n, int w, const int32_t* perm, const double* in, double* out);
 void launch_gather_rows_d(cudaStream_t st, int64_t n, int w, const int32_t* perm, const double* in, double* out);
 void launch_gather_i32(cudaStream_t st, int64_t n, const int32_t* perm, const int32_t* in, int32_t* out);

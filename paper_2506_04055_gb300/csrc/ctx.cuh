@@ -15,7 +15,7 @@ struct DBuf {
   size_t need = 0;   // bytes the last request asked for (the rest of `bytes` is growth headroom)
 };
 
-constexpr int kPartials = 152 * 4;   // fixed block count of the reductions (deterministic)
+constexpr int kPartials = 152 * 4;   // most blocks of the reductions (a function of the atom count: deterministic)
 
 bool bf16_available();
 uint16_t to_bf16_bits(float f);

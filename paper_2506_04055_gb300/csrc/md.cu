@@ -163,7 +163,9 @@ __device__ __forceinline__ void sum_column(int nb, int width, int c, const doubl
   ss[tid] = s;
   sc[tid] = comp;
   __syncthreads();
-  for (int h = kSumThreads / 2; h > 0; h >>= 1) {
+  int h = kSumThreads / 2;
+  while (h >= nb && h > 0) h >>= 1;   // beyond the partials there are only zeros
+  for (; h > 0; h >>= 1) {
     if (tid < h) {
       const double a = ss[tid], b = ss[tid + h], t = a + b;
       const double e = fabs(a) >= fabs(b) ? (a - t) + b : (b - t) + a;
@@ -184,16 +186,6 @@ __global__ void __launch_bounds__(kSumThreads) k_sum_energy_virial(int nb, const
                                                                    double* __restrict__ w) {
   if (blockIdx.x == 0) sum_column(nb, 1, 0, epart, e, 1.0);
   else sum_column(nb, 9, blockIdx.x - 1, vpart, w + blockIdx.x - 1, 1.0);
-}
-
-// out[perm[k]] = (double) in[k]  for [n][w] rows
-__global__ void k_scatter_rows(int64_t n, int w, const int32_t* __restrict__ perm, const float* __restrict__ in,
-                               double* __restrict__ out) {
-  int64_t idx = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (idx >= n * w) return;
-  int64_t k = idx / w;
-  int c = (int)(idx % w);
-  out[(int64_t)perm[k] * w + c] = (double)in[idx];
 }
 
 // out[perm[k]] = in[k]  (double rows) and the inverse gather
@@ -227,6 +219,22 @@ __global__ void k_check_finite(int64_t n, const double* __restrict__ a, int* sta
   int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (k >= n) return;
   if (!isfinite(a[k])) atomicOr(status, (int)ST_NONFINITE);
+}
+
+// A call's outputs in one launch: forces and per-atom energies (either may be null) to the caller's order in FP64,
+// and the report of a non-finite energy or force.
+__global__ void k_outputs(int64_t n, const int32_t* __restrict__ perm, const float* __restrict__ force_s,
+                          const float* __restrict__ eatom, const double* __restrict__ energy, double* __restrict__ force,
+                          double* __restrict__ energies, int* status) {
+  const int64_t idx = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  bool bad = idx == 0 && !isfinite(energy[0]);
+  if (force && idx < 3 * n) {
+    const float f = force_s[idx];
+    force[3 * (int64_t)perm[idx / 3] + idx % 3] = (double)f;
+    bad = bad || !isfinite(f);
+  }
+  if (energies && idx < n) energies[perm[idx]] = (double)eatom[idx];
+  if (bad) atomicOr(status, (int)ST_NONFINITE);
 }
 
 static inline unsigned nblk(int64_t w) { return (unsigned)((w + kThreads - 1) / kThreads); }
@@ -268,12 +276,15 @@ void launch_sum_partials(cudaStream_t st, int nb, int width, const double* parti
   if (width < 1) return;
   { LaunchScope ls_(st); k_sum_partials<<<width, kSumThreads, 0, st>>>(nb, width, partials, out, scale); }
 }
+void launch_outputs(cudaStream_t st, int64_t n, const int32_t* perm, const float* force_s, const float* eatom,
+                    const double* energy, double* force, double* energies, int* status) {
+  const int64_t w = force ? 3 * n : energies ? n : 0;
+  LaunchScope ls_(st);
+  k_outputs<<<nblk(w > 0 ? w : 1), kThreads, 0, st>>>(n, perm, force_s, eatom, energy, force, energies, status);
+}
 void launch_sum_energy_virial(cudaStream_t st, int nb, const double* epart, const double* vpart, double* e, double* w) {
   LaunchScope ls_(st);
   k_sum_energy_virial<<<10, kSumThreads, 0, st>>>(nb, epart, vpart, e, w);
-}
-void launch_scatter_rows(cudaStream_t st, int64_t n, int w, const int32_t* perm, const float* in, double* out) {
-  if (n) { LaunchScope ls_(st); k_scatter_rows<<<nblk(n * w), kThreads, 0, st>>>(n, w, perm, in, out); }
 }
 void launch_scatter_rows_d(cudaStream_t st, int64_t n, int w, const int32_t* perm, const double* in, double* out) {
   if (n) { LaunchScope ls_(st); k_scatter_rows_d<<<nblk(n * w), kThreads, 0, st>>>(n, w, perm, in, out); }
