@@ -110,8 +110,8 @@ int64_t carve(const LocalW& w, int64_t n, int64_t E, float* base, LocalBufs* b) 
     b->gs[q] = cv.take(E * C);
     b->gv[q] = cv.take(E * 3 * C);
   }
-  b->gom = cv.take(E * C2);
-  b->gw0 = cv.take(E * C2);
+  b->gom = cv.take(w.bf16 ? 0 : E * C2);
+  b->gw0 = cv.take(w.bf16 ? 0 : E * C2);
   b->gin = cv.take(E * w.KA);
   b->gg = reinterpret_cast<float4*>(cv.take(E * 4));
   b->ggamS = cv.take(n * C);
@@ -573,7 +573,8 @@ __global__ void k_loc_tp_bwd_atom(int64_t n, int C, const int32_t* __restrict__ 
 // Environment sums, reversed: g_om[c] = f_c g_Gs[c], g_om[C+c] = f_c (g_Gv[c] . u);
 // dE/df_c += om[c] g_Gs[c] + om[C+c] (g_Gv[c] . u);  dE/du += f_c om[C+c] g_Gv[c].
 // Four lanes per edge, each over channel quads j, j + 4, ... (16-byte accesses; C a multiple of 4,
-// of 16 when gomb is written), the sums over channels by two shuffle steps in a fixed order.
+// of 16 when gomb is written), the sums over channels by two shuffle steps in a fixed order.  The
+// BF16 path writes only the GEMM's BF16 operand gomb.
 __global__ void k_loc_env_bwd(int64_t E, int C, const int32_t* __restrict__ erow, const float* __restrict__ geo,
                               const float* __restrict__ om, const float* __restrict__ ggamS,
                               const float* __restrict__ ggamV, float* __restrict__ gom, float4* __restrict__ gg,
@@ -607,11 +608,12 @@ __global__ void k_loc_env_bwd(int64_t E, int C, const int32_t* __restrict__ erow
     one(gs.y, q0.y, q1.y, q2.y, o0.y, o1.y, va.y, vb.y);
     one(gs.z, q0.z, q1.z, q2.z, o0.z, o1.z, va.z, vb.z);
     one(gs.w, q0.w, q1.w, q2.w, o0.w, o1.w, va.w, vb.w);
-    *reinterpret_cast<float4*>(gom + es * 2 * C + c) = va;
-    *reinterpret_cast<float4*>(gom + es * 2 * C + C + c) = vb;
     if (gomb) {
       st4_bf16(gomb + es * Kc + c, va);
       st4_bf16(gomb + es * Kc + C + c, vb);
+    } else {
+      *reinterpret_cast<float4*>(gom + es * 2 * C + c) = va;
+      *reinterpret_cast<float4*>(gom + es * 2 * C + C + c) = vb;
     }
   }
   if (live && gomb)
@@ -650,11 +652,12 @@ __global__ void k_loc_init_bwd(int64_t E, int C, const float* __restrict__ w0, c
     const float4 va = ld4f(GS + es * C + c), wv = ld4f(w0 + es * 2 * C + C + c);
     const float4 vb = make_float4(fmaf(q2.x, u2, fmaf(q1.x, u1, q0.x * u0)), fmaf(q2.y, u2, fmaf(q1.y, u1, q0.y * u0)),
                                   fmaf(q2.z, u2, fmaf(q1.z, u1, q0.z * u0)), fmaf(q2.w, u2, fmaf(q1.w, u1, q0.w * u0)));
-    *reinterpret_cast<float4*>(gw0 + es * 2 * C + c) = va;
-    *reinterpret_cast<float4*>(gw0 + es * 2 * C + C + c) = vb;
     if (gw0b) {
       st4_bf16(gw0b + es * Kc + c, va);
       st4_bf16(gw0b + es * Kc + C + c, vb);
+    } else {
+      *reinterpret_cast<float4*>(gw0 + es * 2 * C + c) = va;
+      *reinterpret_cast<float4*>(gw0 + es * 2 * C + C + c) = vb;
     }
     gu0 = fmaf(wv.w, q0.w, fmaf(wv.z, q0.z, fmaf(wv.y, q0.y, fmaf(wv.x, q0.x, gu0))));
     gu1 = fmaf(wv.w, q1.w, fmaf(wv.z, q1.z, fmaf(wv.y, q1.y, fmaf(wv.x, q1.x, gu1))));
