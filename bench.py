@@ -400,7 +400,8 @@ def run_ours(args):
         launch_s = dom_ms / dom_launches / 1e3
         tc = head == "bf16" and F == 128 and ((dom == "edge_fwd" and args.tc_message != 0) or
                                               (dom == "edge_bwd" and args.tc_adjoint != 0))
-        kname = ("k_edge_bwd_tcg" if dom == "edge_bwd" else "k_edge_msg_mma") if tc else f"k_{dom}"
+        kname = (("k_edge_bwd_tcg" if dom == "edge_bwd" else "k_edge_msg_mma") if tc else
+                 ("k_edge_adj" if dom == "edge_bwd" else "k_edge_msg"))
         flop = ea * edge_flop_per_edge()
         achieved = flop / launch_s / 1e12
         if tc:
