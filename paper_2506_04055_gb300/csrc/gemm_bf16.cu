@@ -234,7 +234,8 @@ __global__ void __launch_bounds__(64 + 32 * epi_warps<EPI>(), 1) k_gemm_bf16(con
               const int r = 3 * al + k, qq = r >> 5;
               const float* Tq = sT + (4 * grp + ((qq + 2) & 3)) * 32 * kTP;
               const float4 t = *reinterpret_cast<const float4*>(Tq + (r & 31) * kTP + fq);
-              const float4 gk = __ldg(reinterpret_cast<const float4*>(p.aux + (3 * ai + k) * p.ldaux + c0 + fq));
+              const float4 gk = p.aux ? __ldg(reinterpret_cast<const float4*>(p.aux + (3 * ai + k) * p.ldaux + c0 + fq))
+                                      : make_float4(0.f, 0.f, 0.f, 0.f);   // aux null: zero
               x[k] = make_float4(t.x + gk.x, t.y + gk.y, t.z + gk.z, t.w + gk.w);
             }
             const float4 gs = __ldg(reinterpret_cast<const float4*>(p.aux2 + ai * p.N + c0 + fq));
@@ -409,7 +410,7 @@ int gemm_bf16(cudaStream_t st, int64_t M, int N, int K, const bf16* A, int64_t l
               int* status, __half* outh, const float* aux2, const __half* auxh) {
   if (M == 0) return 0;
   // EPI 5: rows (atom, component) of whole atoms, 32-bit row arithmetic in the epilogue
-  if (EPI == 5 && (M % 3 != 0 || M >= ((int64_t)1 << 31) || !out || !aux || !aux2 ||
+  if (EPI == 5 && (M % 3 != 0 || M >= ((int64_t)1 << 31) || !out || !aux2 ||
                    (reinterpret_cast<uintptr_t>(aux2) & 15)))
     return -1;
   // the epilogue moves 16-byte quads of FP32 (8-byte quads of BF16) per row

@@ -304,7 +304,8 @@ __global__ void k_embed(int64_t n, int F, const int32_t* __restrict__ Z, const f
   }
 }
 
-// PHI[i] = [phi_s | v_0 phi_vv | v_1 phi_vv | v_2 phi_vv | phi_vs | phi_vv]
+// PHI[i] = [phi_s | v_0 phi_vv | v_1 phi_vv | v_2 phi_vv | phi_vs | phi_vv]; V null (first layer, v = 0): only
+// phi_s and phi_vs, all that the first layer's edge kernels read
 __global__ void k_phi_pack(int64_t n, int F, const float* __restrict__ P3, const float* __restrict__ V,
                            float* __restrict__ PHI) {
   int64_t idx = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
@@ -312,8 +313,13 @@ __global__ void k_phi_pack(int64_t n, int F, const float* __restrict__ P3, const
   int64_t i = idx / F;
   int f = (int)(idx % F);
   const float* p = P3 + i * 3 * F;
-  const float* v = V + i * 3 * F;
   float* o = PHI + i * 6 * F;
+  if (!V) {
+    o[f] = p[f];
+    o[4 * F + f] = p[2 * F + f];
+    return;
+  }
+  const float* v = V + i * 3 * F;
   float pvv = p[F + f];
   o[f] = p[f];
   o[F + f] = v[f] * pvv;
@@ -422,7 +428,7 @@ __global__ void k_update_bwd_pre(int64_t n, int F, const float* __restrict__ GS,
 #pragma unroll
   for (int al = 0; al < 3; ++al) {
     float u = uv[al * 2 * F + f], v = uv[al * 2 * F + F + f];
-    float gv = GV[i * 3 * F + al * F + f];
+    float gv = GV ? GV[i * 3 * F + al * F + f] : 0.0f;   // null: the last layer, whose v reaches nothing
     sp += u * v;
     gavv += gv * u;
     GUV[i * 6 * F + al * 2 * F + f] = gv * avv + gsp * v;
@@ -480,7 +486,7 @@ __global__ void k_update_bwd_pre_bf16(int64_t n, int F, const float* __restrict_
 #pragma unroll
   for (int al = 0; al < 3; ++al) {
     const float u = ldx(uv + al * 2 * F + f), v = ldx(uv + al * 2 * F + F + f);
-    const float gv = GV[i * 3 * F + al * F + f];
+    const float gv = GV ? GV[i * 3 * F + al * F + f] : 0.0f;
     sp += u * v;
     gavv += gv * u;
     GUVb[i * 6 * F + al * 2 * F + f] = __float2bfloat16_rn(gv * avv + gsp * v);
@@ -990,10 +996,12 @@ void model_forward_backward_fp32(cudaStream_t st, const ModelW& m, int64_t n, co
   StageGuard node_stage(STG_NODE);
   const int F = m.F, T = m.T;
   const unsigned nb = blocks_for(n * F), nb4 = blocks_for(n * F / 4);   // nb4: four features per thread
-  if (n > 0) { LaunchScope ls_(st); k_embed<<<nb, kThreads, 0, st>>>(n, F, species_s, m.emb, B[B_S0], B[B_V0], nullptr); }
+  // the first layer's v = 0 is stored and read only where its filters are stored
+  float* v0 = wstore && need_grad ? B[B_V0] : nullptr;
+  if (n > 0) { LaunchScope ls_(st); k_embed<<<nb, kThreads, 0, st>>>(n, F, species_s, m.emb, B[B_S0], v0, nullptr); }
   for (int t = 0; t < T; ++t) {
     const LayerW& L = m.L[t];
-    float *S = B[B_S0], *V = B[B_V0 + t], *PHI = B[B_PHI0 + t], *H1 = B[B_H10 + t];
+    float *S = B[B_S0], *V = t == 0 ? v0 : B[B_V0 + t], *PHI = B[B_PHI0 + t], *H1 = B[B_H10 + t];
     float *SM = B[B_SM0], *VM = B[B_VM0], *UV = B[B_UV0 + t], *H2 = B[B_H20 + t], *AV = B[B_AV0 + t];
     float *T1 = B[B_T1], *T2 = B[B_T2];
     // phi = W2 silu(W1 s + b1) + b2
@@ -1024,19 +1032,20 @@ void model_forward_backward_fp32(cudaStream_t st, const ModelW& m, int64_t n, co
   // readout, and dU/ds^T = G3 R1
   readout_fwd_bwd(st, m, n, B[B_S0], ew, need_grad, B, e_atom, energy_partials, n_energy_partials);
   if (!need_grad) return;
-  if (n > 0) cudaMemsetAsync(B[B_GV], 0, sizeof(float) * (size_t)n * 3 * F, st);
   for (int t = T - 1; t >= 0; --t) {
     const LayerW& L = m.L[t];
     float *V = B[B_V0 + t], *PHI = B[B_PHI0 + t], *H1 = B[B_H10 + t];
     float *UV = B[B_UV0 + t], *H2 = B[B_H20 + t], *AV = B[B_AV0 + t];
     float *T1 = B[B_T1], *T2 = B[B_T2], *T3 = B[B_T3];
     float *GS = B[B_GS], *GV = B[B_GV], *GSM = B[B_GSM], *GVM = B[B_GVM], *GPHI = B[B_GPHI];
+    const float* gvn = t == T - 1 ? nullptr : GV;   // gradient of the layer's v: the last one's is zero
     // update backward
-    if (n > 0) { LaunchScope ls_(st); k_update_bwd_pre<<<nb, kThreads, 0, st>>>(n, F, GS, GV, UV, AV, T1, T3, nullptr); }
+    if (n > 0) { LaunchScope ls_(st); k_update_bwd_pre<<<nb, kThreads, 0, st>>>(n, F, GS, gvn, UV, AV, T1, T3, nullptr); }
     gemm<EPI_DSILU>(st, n, F, 3 * F, T1, 3 * F, L.A2, nullptr, H2, F, T2, F);          // gh2
     gemm<EPI_BIAS>(st, n, 2 * F, F, T2, F, L.A1, nullptr, nullptr, 0, T1, 2 * F);       // gz
     if (n > 0) { LaunchScope ls_(st); k_update_bwd_mid<<<nb, kThreads, 0, st>>>(n, F, m.eps, GS, T1, UV, GSM, T3, nullptr); }
-    gemm<EPI_ADD>(st, 3 * n, F, 2 * F, T3, 2 * F, L.UV, nullptr, GV, F, GVM, F);         // gvm
+    if (gvn) gemm<EPI_ADD>(st, 3 * n, F, 2 * F, T3, 2 * F, L.UV, nullptr, gvn, F, GVM, F);   // gvm
+    else gemm<EPI_BIAS>(st, 3 * n, F, 2 * F, T3, 2 * F, L.UV, nullptr, nullptr, 0, GVM, F);
     // message backward
     const float* wst = wstore ? wstore + t * wstore_layer_floats : nullptr;
     // the first layer's inputs (embedding, v = 0) do not depend on positions: its edge adjoint
@@ -1186,7 +1195,6 @@ int model_forward_backward_bf16(cudaStream_t st, const ModelW& m, int64_t n, con
   // per-atom energy itself, which BF16 operands would perturb by ~2^-9 of the readout terms.
   readout_fwd_bwd(st, m, n, B[B_S0], ew, need_grad, B, e_atom, energy_partials, n_energy_partials);
   if (!need_grad) return bad;
-  if (n > 0) cudaMemsetAsync(B[B_GV], 0, sizeof(float) * (size_t)n * 3 * F, st);
   for (int t = T - 1; t >= 0; --t) {
     const LayerW& L = m.L[t];
     float *V = B[B_V0 + t], *PHI = phi32 ? B[B_PHI0 + t] : nullptr;
@@ -1196,8 +1204,9 @@ int model_forward_backward_bf16(cudaStream_t st, const ModelW& m, int64_t n, con
     const __half* AV = reinterpret_cast<const __half*>(Bb[BB_AVH0 + t]);
     float* T1 = B[B_T1];
     float *GS = B[B_GS], *GV = B[B_GV], *GSM = B[B_GSM], *GVM = B[B_GVM], *GPHI = B[B_GPHI];
+    const float* gvn = t == T - 1 ? nullptr : GV;   // gradient of the layer's v: the last one's is zero
     const __half* PHIh = phih(t);
-    if (n > 0) { LaunchScope ls_(st); k_update_bwd_pre_bf16<<<nb, kThreads, 0, st>>>(n, F, GS, GV, UV, AV, Bb[BB_GA], Bb[BB_GUV]); }
+    if (n > 0) { LaunchScope ls_(st); k_update_bwd_pre_bf16<<<nb, kThreads, 0, st>>>(n, F, GS, gvn, UV, AV, Bb[BB_GA], Bb[BB_GUV]); }
     bad |= gemm_bf16<6>(st, n, F, 3 * F, Bb[BB_GA], 3 * F, L.A2tb, nullptr, nullptr, F, nullptr, 0, Bb[BB_GH2], F, status,
                         nullptr, nullptr, H2);
     bad |= gemm_bf16<0>(st, n, 2 * F, F, Bb[BB_GH2], F, L.A1tb, nullptr, nullptr, 0, T1, 2 * F, nullptr, 0, status);
@@ -1205,8 +1214,10 @@ int model_forward_backward_bf16(cudaStream_t st, const ModelW& m, int64_t n, con
     float* G4 = g4 ? B[B_G4] : nullptr;
     if (n > 0) { LaunchScope ls_(st); k_update_bwd_mid_bf16<<<nb4, kThreads, 0, st>>>(n, F, m.eps, GS, T1, UV, AV, GSM, Bb[BB_GUV]); }
     if (G4)   // gvm = gv + the U/V backward, written straight into G4 beside gsm
-      bad |= gemm_bf16<5>(st, 3 * n, F, 2 * F, Bb[BB_GUV], 2 * F, L.UVtb, nullptr, GV, F, G4, F, nullptr, 0, status,
+      bad |= gemm_bf16<5>(st, 3 * n, F, 2 * F, Bb[BB_GUV], 2 * F, L.UVtb, nullptr, gvn, F, G4, F, nullptr, 0, status,
                           nullptr, GSM);
+    else if (!gvn)
+      bad |= gemm_bf16<0>(st, 3 * n, F, 2 * F, Bb[BB_GUV], 2 * F, L.UVtb, nullptr, nullptr, 0, GVM, F, nullptr, 0, status);
     else
       bad |= gemm_bf16<2>(st, 3 * n, F, 2 * F, Bb[BB_GUV], 2 * F, L.UVtb, nullptr, GV, F, GVM, F, nullptr, 0, status);
     const float* wst = (wstore && !use_tc_bwd && !msg_mma) ? wstore + t * wstore_layer_floats : nullptr;
