@@ -138,7 +138,7 @@ __device__ __forceinline__ void cp_async_wait() {
 // flight at once with cp.async, in 64-deep commit groups, and the chain over k starts as soon as
 // the first group has landed: one memory latency per launch.  The thread-per-output kernel that
 // stood here walked K with a global load per step (192 atoms, F = 64: 13 to 33 us per launch, now
-// 4.4 to 7.3; 5,997 atoms: 23 to 47 us, now 8 to 15).
+// 2.6 to 5.6; 5,997 atoms: 23 to 47 us, now 6 to 12).
 // Same fmaf chain over k in increasing order and same epilogue as k_gemm: bit-identical outputs.
 constexpr int GSK = 64;   // k per commit group
 template <int BM, int BN>
