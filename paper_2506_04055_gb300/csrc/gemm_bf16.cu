@@ -1,11 +1,12 @@
 // gemm_bf16.cu -- persistent tcgen05 GEMM for the node MLPs of the BF16 path:
 //   C[M][N] = A[M][K] . W[N][K]^T   (BF16 operands, FP32 accumulation in TMEM)
 // with the same fused epilogues as the FP32 SIMT GEMM (bias, bias + SiLU, residual add,
-// multiply by SiLU') and one that packs the phi-MLP output into the message kernel's PHI rows.  A rows are atoms (or atom x spatial component), W is a weight matrix
-// stored [out][in], i.e. K-major, so both operands are K-major 128B-swizzled tiles.
+// multiply by SiLU') and one that packs the phi-MLP output into the message kernel's PHI rows.  A
+// rows are atoms (or atom x spatial component), W is a weight matrix stored [out][in], i.e. K-major, so both operands are K-major 128B-swizzled tiles.
 //
-// One CTA per SM (persistent over 128-row tiles).  Warp 0: TMA producer (the weight tile W is
-// loaded once per CTA and stays in shared memory; A streams through a ring of 64-column
+// One CTA per SM (persistent over 128-row tiles; few tiles are shared by several CTAs, each with its
+// share of the columns).  Warp 0: TMA producer (the CTA's rows of W are
+// loaded once and stays in shared memory; A streams through a ring of 64-column
 // k-blocks, 16 KB each, as many stages as shared memory holds).  Warp 1: TMEM allocation and
 // the single-thread MMA issue (M = 128, N up to 256 per instruction, K = 16 per instruction).
 // Warps 2 and up: epilogue, epi_warps / 4 warps per TMEM lane quarter taking the quarter's
