@@ -6,7 +6,7 @@
 //
 // One CTA per SM (persistent over 128-row tiles; few tiles are shared by several CTAs, each with its
 // share of the columns).  Warp 0: TMA producer (the CTA's rows of W are
-// loaded once and stays in shared memory; A streams through a ring of 64-column
+// loaded once and stay in shared memory; A streams through a ring of 64-column
 // k-blocks, 16 KB each, as many stages as shared memory holds).  Warp 1: TMEM allocation and
 // the single-thread MMA issue (M = 128, N up to 256 per instruction, K = 16 per instruction).
 // Warps 2 and up: epilogue, epi_warps / 4 warps per TMEM lane quarter taking the quarter's
