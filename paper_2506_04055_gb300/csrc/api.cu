@@ -266,18 +266,29 @@ int prune_begin(ctd_ctx* c, double* maxdisp_out) {
   return CTD_OK;
 }
 
-// ... and the active list itself.
-int prune_finish(ctd_ctx* c) {
-  StageGuard sg(STG_PRUNE);
-  cudaStream_t st = c->st;
-  const int64_t n = c->n, n1 = n > 0 ? n : 1, e1 = c->n_verlet > 0 ? c->n_verlet : 1;
-  ENSURE(c, c->acount, sizeof(int32_t) * n1);
-  ENSURE(c, c->arow, sizeof(int32_t) * (n1 + 1));
+// The buffers of a forces step whose size follows the Verlet list.  Grown by every step before its work
+// is recorded or replayed: a replay runs no checks, and a list may have been built (by a call that only
+// builds, or by one that failed after its build) since these were last sized.
+int ensure_edge_buffers(ctd_ctx* c) {
+  const int64_t e1 = c->n_verlet > 0 ? c->n_verlet : 1;
   ENSURE(c, c->acol, sizeof(int32_t) * e1);
   ENSURE(c, c->ar, sizeof(float4) * e1);
   ENSURE(c, c->vidx, sizeof(int32_t) * e1);
   ENSURE(c, c->arev, sizeof(int32_t) * e1);
   ENSURE(c, c->aend, sizeof(int32_t) * e1);
+  ENSURE(c, c->hedge, sizeof(float4) * e1);
+  return CTD_OK;
+}
+
+// ... and the active list itself.
+int prune_finish(ctd_ctx* c) {
+  StageGuard sg(STG_PRUNE);
+  cudaStream_t st = c->st;
+  const int64_t n = c->n, n1 = n > 0 ? n : 1;
+  ENSURE(c, c->acount, sizeof(int32_t) * n1);
+  ENSURE(c, c->arow, sizeof(int32_t) * (n1 + 1));
+  const int r = ensure_edge_buffers(c);
+  if (r) return r;
   const float rc2 = (float)(c->desc.rc * c->desc.rc);
   const uint8_t* near = c->use_near ? P<uint8_t>(c->near) : nullptr;
   launch_prune(st, false, n, P<int32_t>(c->vrow), P<int32_t>(c->vcol), P<float4>(c->vbase), P<float4>(c->delta),
@@ -449,8 +460,8 @@ void drop_graph(ctd_ctx* c) {
 // state keeps them sorted) and model.  It has no host decision in it, and below a few ten thousand atoms its
 // seventy launches take the host longer than the device, so it is recorded as a CUDA graph and replayed
 // while everything it bakes in besides device memory contents stays the same: the buffers (by their
-// allocation generation), the atom count, the model options and what is asked for.  The first call of
-// a key runs eagerly (and grows what it needs), the second records; new parameters drop the graph.
+// allocation generation, once those sized by the list are large enough for it), the atom count, the model
+// options and what is asked for.  The first call of a key runs eagerly (and grows what it needs), the second records; new parameters drop the graph.
 // Larger systems gain nothing (96,000 atoms: the device is never idle) and stay eager, as do the
 // strictly local family (it reads its edge count back), stored filters, models without layers (a memset
 // sized by the Verlet list) and profiled calls (events around each launch).
@@ -472,6 +483,8 @@ int forces_step(ctd_ctx* c, bool need_grad, bool gather_z) {
   if (c->local() || c->n == 0 || c->desc.T == 0 || c->n * c->desc.F > kGraphFeatures || prof_recording() ||
       model_stores_edges(c->mw, c->desc.precision))
     return body();
+  const int grown = ensure_edge_buffers(c);   // before the key: growth changes it
+  if (grown) return grown;
   const uint64_t key = key_now();
   if (!(c->gexec && c->gkey == key) && key == c->glast) {
     drop_graph(c);

@@ -118,6 +118,7 @@ int setup_geometry_into(ctd_ctx* c, CellGeom& g, int64_t* ncell, const double H[
 int check_status(ctd_ctx* c);
 int copy_in(ctd_ctx* c, void* dst, const void* src, size_t bytes, bool device);
 int prune(ctd_ctx* c, double* maxdisp_out);
+int ensure_edge_buffers(ctd_ctx* c);
 void drop_graph(ctd_ctx* c);
 int evaluate(ctd_ctx* c, bool need_grad);
 size_t model_bytes_per_atom(const ctd_ctx* c);
