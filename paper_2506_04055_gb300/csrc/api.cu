@@ -450,21 +450,16 @@ int evaluate(ctd_ctx* c, bool need_grad) {
   return CTD_OK;
 }
 
-void drop_graph(ctd_ctx* c) {
-  if (c->gexec) cudaGraphExecDestroy(c->gexec);
-  c->gexec = nullptr;
-  c->gkey = c->glast = 0;
-}
-
 // The device work after the rebuild decision: active list, species (gather_z: of a new call; an MD
-// state keeps them sorted) and model.  It has no host decision in it, and below a few ten thousand atoms its
-// seventy launches take the host longer than the device, so it is recorded as a CUDA graph and replayed
-// while everything it bakes in besides device memory contents stays the same: the buffers (by their
-// allocation generation, once those sized by the list are large enough for it), the atom count, the model
-// options and what is asked for.  The first call of a key runs eagerly (and grows what it needs), the second records; new parameters drop the graph.
-// Larger systems gain nothing (96,000 atoms: the device is never idle) and stay eager, as do the
-// strictly local family (it reads its edge count back), stored filters, models without layers (a memset
-// sized by the Verlet list) and profiled calls (events around each launch).
+// state keeps them sorted) and model.  It has no host decision in it, so it is recorded as a CUDA graph and
+// replayed while everything it bakes in besides device memory contents stays the same: the buffers
+// (by their allocation generation, once those sized by the list are large enough for it), the atom count, the
+// model options and what is asked for.  step_records.h says which keys are recorded; new parameters drop
+// all recordings.  A replay saves about 150 us of gaps between some seventy launches at every size measured (192 atoms
+// 571 -> 420 us, 32,000 at F = 128 6715 -> 6562, 96,000 at F = 64 10933 -> 10788): above kGraphFeatures, where that is
+// below 4 % of a call, steps stay eager, as do those of the strictly local family (it reads its edge
+// count back), stored filters, models without layers (a memset sized by the Verlet list) and profiled
+// calls (events around each launch).
 int forces_step(ctd_ctx* c, bool need_grad, bool gather_z) {
   auto body = [&]() -> int {
     const int r = prune_finish(c);
@@ -485,9 +480,11 @@ int forces_step(ctd_ctx* c, bool need_grad, bool gather_z) {
     return body();
   const int grown = ensure_edge_buffers(c);   // before the key: growth changes it
   if (grown) return grown;
+  using Act = decltype(c->records)::Act;
   const uint64_t key = key_now();
-  if (!(c->gexec && c->gkey == key) && key == c->glast) {
-    drop_graph(c);
+  Act act = c->records.next(key);
+  if (act == Act::kRecord) {
+    auto* rec = new RecordedStep();
     cudaGraph_t g = nullptr;
     int64_t before[STG_COUNT];
     for (int k = 0; k < STG_COUNT; ++k) before[k] = c->prof.launches[k];
@@ -498,27 +495,29 @@ int forces_step(ctd_ctx* c, bool need_grad, bool gather_z) {
       if (cudaStreamEndCapture(c->st, &g) != cudaSuccess) r = CTD_ERR_CUDA;
     }
     c->capturing = false;
-    if (r == CTD_OK && g && key_now() == key && cudaGraphInstantiate(&c->gexec, g, 0) == cudaSuccess) {
-      c->gkey = key;
+    for (int k = 0; k < STG_COUNT; ++k) {   // counted when the graph is launched
+      rec->launches[k] = c->prof.launches[k] - before[k];
+      c->prof.launches[k] = before[k];
+    }
+    if (r == CTD_OK && g && key_now() == key && cudaGraphInstantiate(&rec->exec, g, 0) == cudaSuccess) {
+      c->records.recorded(key, rec);
+      act = Act::kReplay;
     } else {
-      c->gexec = nullptr;
+      delete rec;
+      c->records.refused(key);
       cudaGetLastError();
       c->err.clear();
     }
     if (g) cudaGraphDestroy(g);
-    for (int k = 0; k < STG_COUNT; ++k) {   // counted when the graph is launched
-      c->glaunches[k] = c->prof.launches[k] - before[k];
-      c->prof.launches[k] = before[k];
-    }
   }
-  if (c->gexec && c->gkey == key) {
-    CUDA_OK(c, cudaGraphLaunch(c->gexec, c->st));
-    for (int k = 0; k < STG_COUNT; ++k) c->prof.launches[k] += c->glaunches[k];
+  if (act == Act::kReplay) {
+    const RecordedStep* rec = c->records.replay(key);
+    CUDA_OK(c, cudaGraphLaunch(rec->exec, c->st));
+    for (int k = 0; k < STG_COUNT; ++k) c->prof.launches[k] += rec->launches[k];
     return CTD_OK;
   }
-  const bool tried = c->glast == key;   // the capture did not complete: not again for this key
   const int r = body();
-  c->glast = r == CTD_OK && !tried ? key_now() : 0;
+  if (r == CTD_OK) c->records.ran(key_now());
   return r;
 }
 
@@ -671,7 +670,7 @@ int load_local_params(ctd_ctx* c, const char* b, size_t nbytes) {
 }
 
 int load_params_impl(ctd_ctx* c, const void* blob, size_t nbytes) {
-  drop_graph(c);
+  c->records.clear();
   if (!blob || nbytes < 64) return fail(c, CTD_ERR_INVALID_ARG, "parameter blob too short");
   const char* b = static_cast<const char*>(blob);
   if (c->local()) return load_local_params(c, b, nbytes);
@@ -886,7 +885,7 @@ int ctd_create(ctd_ctx** out, const ctd_model_desc* desc, size_t hbm_budget_byte
 void ctd_destroy(ctd_ctx* c) {
   if (!c) return;
   if (c->st) cudaStreamSynchronize(c->st);
-  drop_graph(c);
+  c->records.clear();
   c->prof.collect();
   for (DBuf* b : c->all)
     if (b->p) cudaFree(b->p);

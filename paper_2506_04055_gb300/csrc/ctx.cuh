@@ -6,6 +6,7 @@
 #include <vector>
 
 #include "ctd_internal.cuh"
+#include "step_records.h"
 #include "../../include/painn.h"
 
 namespace ctd {
@@ -13,6 +14,18 @@ struct DBuf {
   void* p = nullptr;
   size_t bytes = 0;
   size_t need = 0;   // bytes the last request asked for (the rest of `bytes` is growth headroom)
+};
+
+// A step recorded as a CUDA graph and the launches it holds per stage.
+struct RecordedStep {
+  cudaGraphExec_t exec = nullptr;
+  int64_t launches[STG_COUNT] = {};
+};
+struct DropRecordedStep {
+  void operator()(RecordedStep* r) const {
+    cudaGraphExecDestroy(r->exec);
+    delete r;
+  }
 };
 
 constexpr int kPartials = 152 * 4;   // most blocks of the reductions (a function of the atom count: deterministic)
@@ -39,11 +52,8 @@ struct ctd_ctx {
   bool capturing = false;
   uint64_t alloc_gen = 0;
   std::vector<DBuf*> all;
-  // recorded forces step of a call or MD step (api.cu, forces_step): its key, the key of the last
-  // eager step, and the launches it holds per stage
-  cudaGraphExec_t gexec = nullptr;
-  uint64_t gkey = 0, glast = 0;
-  int64_t glaunches[ctd::STG_COUNT] = {};
+  // recorded forces steps of calls and MD steps (api.cu, forces_step)
+  ctd::StepRecords<ctd::RecordedStep*, ctd::DropRecordedStep> records;
 
   // parameters
   bool have_params = false;
@@ -119,7 +129,6 @@ int check_status(ctd_ctx* c);
 int copy_in(ctd_ctx* c, void* dst, const void* src, size_t bytes, bool device);
 int prune(ctd_ctx* c, double* maxdisp_out);
 int ensure_edge_buffers(ctd_ctx* c);
-void drop_graph(ctd_ctx* c);
 int evaluate(ctd_ctx* c, bool need_grad);
 size_t model_bytes_per_atom(const ctd_ctx* c);
 
