@@ -488,18 +488,12 @@ int forces_step(ctd_ctx* c, bool need_grad, bool gather_z) {
     cudaGraph_t g = nullptr;
     int64_t before[STG_COUNT];
     for (int k = 0; k < STG_COUNT; ++k) before[k] = c->prof.launches[k];
-    c->capturing = true;
-    int r = CTD_ERR_CUDA;
-    if (cudaStreamBeginCapture(c->st, cudaStreamCaptureModeThreadLocal) == cudaSuccess) {
-      r = body();
-      if (cudaStreamEndCapture(c->st, &g) != cudaSuccess) r = CTD_ERR_CUDA;
-    }
-    c->capturing = false;
+    const int r = record_graph(c, body, &g);
     for (int k = 0; k < STG_COUNT; ++k) {   // counted when the graph is launched
       rec->launches[k] = c->prof.launches[k] - before[k];
       c->prof.launches[k] = before[k];
     }
-    if (r == CTD_OK && g && key_now() == key && cudaGraphInstantiate(&rec->exec, g, 0) == cudaSuccess) {
+    if (r == CTD_OK && key_now() == key && cudaGraphInstantiate(&rec->exec, g, 0) == cudaSuccess) {
       c->records.recorded(key, rec);
       act = Act::kReplay;
     } else {
@@ -893,6 +887,7 @@ void ctd_destroy(ctd_ctx* c) {
     if (b.p) cudaFree(b.p);
   for (DBuf& b : c->mbufb)
     if (b.p) cudaFree(b.p);
+  if (c->capture_st) cudaStreamDestroy(c->capture_st);
   if (c->own_stream) cudaStreamDestroy(c->st);
   delete c;
 }

@@ -3,6 +3,7 @@
 // calls (api.cu) and the multi-replica serving loop (serve.cu).
 #pragma once
 #include <string>
+#include <utility>
 #include <vector>
 
 #include "ctd_internal.cuh"
@@ -43,6 +44,7 @@ struct ctd_ctx {
   ctd_model_desc desc{};
   int device = 0;
   cudaStream_t st = nullptr;
+  cudaStream_t capture_st = nullptr;   // recordings are made here (record_graph)
   bool own_stream = false;
   size_t budget = 0, held = 0, used = 0;   // used: the buffers' last requests
   std::string err;
@@ -129,6 +131,32 @@ int check_status(ctd_ctx* c);
 int copy_in(ctd_ctx* c, void* dst, const void* src, size_t bytes, bool device);
 int prune(ctd_ctx* c, double* maxdisp_out);
 int ensure_edge_buffers(ctd_ctx* c);
+// Records what `body` puts on c->st (kernels and memsets, no host decisions) as a graph instead of running
+// it; CTD_OK and *graph, or an error with nothing recorded.  The recording is made on a stream of the
+// context's own: while a stream is being captured, whatever another thread puts on it is captured
+// too, and a stream passed in by the caller may be shared, or may not allow capture at all.
+template <class Body>
+int record_graph(ctd_ctx* c, Body&& body, cudaGraph_t* graph) {
+  *graph = nullptr;
+  if (!c->capture_st && cudaStreamCreateWithFlags(&c->capture_st, cudaStreamNonBlocking) != cudaSuccess) {
+    c->capture_st = nullptr;
+    return CTD_ERR_CUDA;
+  }
+  int r = CTD_ERR_CUDA;
+  if (cudaStreamBeginCapture(c->capture_st, cudaStreamCaptureModeThreadLocal) == cudaSuccess) {
+    c->capturing = true;
+    std::swap(c->st, c->capture_st);
+    r = body();
+    std::swap(c->st, c->capture_st);
+    c->capturing = false;
+    if (cudaStreamEndCapture(c->capture_st, graph) != cudaSuccess) r = CTD_ERR_CUDA;
+  }
+  if (r != CTD_OK && *graph) {
+    cudaGraphDestroy(*graph);
+    *graph = nullptr;
+  }
+  return r;
+}
 int evaluate(ctd_ctx* c, bool need_grad);
 size_t model_bytes_per_atom(const ctd_ctx* c);
 

@@ -588,14 +588,8 @@ bool capture_step(ctd_server* s, int64_t nres, uint64_t key) {
   ctd_ctx* c = s->c;
   drop_graph(s);
   cudaGraph_t g = nullptr;
-  c->capturing = true;
-  int r = CTD_ERR_CUDA;
-  if (cudaStreamBeginCapture(c->st, cudaStreamCaptureModeThreadLocal) == cudaSuccess) {
-    r = step_device(s, nres);
-    if (cudaStreamEndCapture(c->st, &g) != cudaSuccess) r = CTD_ERR_CUDA;
-  }
-  c->capturing = false;
-  bool ok = r == CTD_OK && g && layout_key(s, nres) == key && cudaGraphInstantiate(&s->gexec, g, 0) == cudaSuccess;
+  const int r = record_graph(c, [&] { return step_device(s, nres); }, &g);
+  bool ok = r == CTD_OK && layout_key(s, nres) == key && cudaGraphInstantiate(&s->gexec, g, 0) == cudaSuccess;
   if (ok) {
     size_t nn = 0;
     cudaGraphGetNodes(g, nullptr, &nn);
