@@ -15,6 +15,7 @@
 #include <vector>
 
 #include "ctx.cuh"
+#include "gauss_reach.h"
 
 using namespace ctd;
 
@@ -805,6 +806,7 @@ int load_params_impl(ctd_ctx* c, const void* blob, size_t nbytes) {
     L.W1 = base + o.W1; L.W1t = base + o.W1t; L.b1 = base + o.b1;
     L.W2 = base + o.W2; L.W2t = base + o.W2t; L.b2 = base + o.b2;
     L.Wf = base + o.Wf; L.bf = base + o.bf;
+    L.reach = gauss_reach(h.data() + o.Wf, 3 * F, KP, K);
     L.UV = base + o.UV; L.UVt = base + o.UVt;
     L.A1 = base + o.A1; L.A1t = base + o.A1t; L.c1 = base + o.c1;
     L.A2 = base + o.A2; L.A2t = base + o.A2t; L.c2 = base + o.c2;

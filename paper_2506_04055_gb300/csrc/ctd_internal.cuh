@@ -90,6 +90,7 @@ struct LayerW {
   const float *W1, *W1t, *b1;      // [F][F]
   const float *W2, *W2t, *b2;      // [3F][F], [F][3F]
   const float *Wf, *bf;            // [3F][KP] (zero padded), [3F]
+  float reach;                     // how many widths below an edge's distance its centres are visited (gauss_reach.h)
   const float *UV, *UVt;           // [2F][F] = [U;V], [F][2F] = [U^T | V^T]
   const float *A1, *A1t, *c1;      // [F][2F], [2F][F]
   const float *A2, *A2t, *c2;      // [3F][F], [F][3F]

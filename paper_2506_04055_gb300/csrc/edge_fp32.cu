@@ -13,13 +13,16 @@
 //     arithmetic rate at half its issue slots: measured 1.9 against 3.9 warp instructions per clock
 //     and SM); in the contraction a packed instruction takes a pair of centres instead, even and odd
 //     centres being added at the end.
-//   * The Gaussians below e^-20 of their peak are not visited.  The basis is ordered by its centres:
-//     every edge takes the last three (K > 20: four) groups of four centres, their weights in
+//   * The Gaussians whose terms are lost in the rounding are not visited.  The basis is ordered by its
+//     centres: every edge takes the last three (K > 20: four) groups of four centres, their weights in
 //     registers, in one straight run of independent chains; an edge takes an earlier group, its
-//     weights in shared memory, only if one of its centres lies within 6.3 widths of the distance
-//     (K = 20 centres over a 5 A cutoff: 14 of 20 centres on average in water and in fcc crystals).
-//     The branch is uniform over the warp.  The terms left out are below 2e-9 of a weight, against
-//     6e-8 for the rounding of one term of the sum.
+//     weights in shared memory, only if one of its centres lies within the layer's reach of the
+//     distance: 6.3 widths or more, worked out from the weights (gauss_reach.h) so that in every channel
+//     and at every distance the terms left out add up to at most 2^-26 of the largest one kept, where
+//     FP32 rounds that one to 2^-24.  Weights of one scale give 6.6 to 7.1 widths (K = 20 centres
+//     over a 5 A cutoff: 14 of 20 centres on average in water and in fcc crystals); far weights that
+//     dwarf the near ones a longer reach, up to every Gaussian that FP32 can tell from zero.  The
+//     branch is uniform over the warp.
 //   * The cutoff is folded into the staged basis (b_k f_c, and its distance derivative for the
 //     adjoint), so the contraction gives W and dW/dd themselves.
 //   * The 32 lanes of a warp stage the next 32 edges at once, across the rows of a chunk of
@@ -95,7 +98,6 @@ __device__ __forceinline__ FV<2> fold(const float2 (&a)[2]) { return {make_float
 constexpr int kStage = 32;             // edges staged at a time, one per lane
 constexpr int kBatch = 8;              // edges whose partials are reduced over the features together
 constexpr int kPartStride = 36;        // float4 per edge of a batch (32 lanes, padded: conflict-free)
-constexpr float kNegligible = 20.0f;   // Gaussians below e^-20 are not visited
 constexpr int64_t kChunkRows = 8;      // consecutive rows a warp group takes at a time, at most
 
 // Groups of four centres, and how many of the last ones keep their weights in registers.
@@ -105,7 +107,7 @@ constexpr int reg_groups() { return KR > 20 ? 4 : 3; }
 struct Args {
   int64_t n, nchunks;
   int K, KP;
-  float rc;
+  float rc, reach;
   int accumulate;
   const int32_t* __restrict__ arow;
   const int32_t* __restrict__ acol;
@@ -149,7 +151,7 @@ __device__ __forceinline__ void stage_edge(const Args& a, float4 r, int col, flo
   const float fc = 0.5f * (cospif(d * inv_rc) + 1.0f);
   const float dfc = GRAD ? -0.5f * 3.14159265358979f * inv_rc * sinpif(d * inv_rc) : 0.0f;
   const float ux = r.x * id, uy = r.y * id, uz = r.z * id;
-  const int first = (int)ceilf((d - sqrtf(2.0f * kNegligible) * sig) / sig);
+  const int first = (int)ceilf((d - a.reach * sig) / sig);
   geo.xy = make_float4(ux, ux, uy, uy);
   geo.zf = make_float4(uz, uz, fc, fc);
   *reinterpret_cast<float4*>(&geo.dfc) =
@@ -694,7 +696,7 @@ void edge_msg_f32(cudaStream_t st, const ModelW& m, int t, int64_t n, const int3
                   __nv_bfloat16* VMb, float* wst) {
   if (n == 0) return;
   Args a{};
-  a.n = n; a.K = m.K; a.KP = m.KP; a.rc = m.rc; a.arow = arow; a.acol = acol; a.ar = ar; a.PHI = PHI;
+  a.n = n; a.K = m.K; a.KP = m.KP; a.rc = m.rc; a.reach = m.L[t].reach; a.arow = arow; a.acol = acol; a.ar = ar; a.PHI = PHI;
   a.Wf = m.L[t].Wf; a.bf = m.L[t].bf; a.S = S; a.V = V; a.SM = SM; a.VM = VM; a.VMb = VMb; a.wst = wst;
   CTD_DISPATCH(msg_go)
 }
@@ -704,7 +706,7 @@ void edge_adj_f32(cudaStream_t st, const ModelW& m, int t, int accumulate, int64
                   float* GPHI, float4* hedge, const float* wst) {
   if (n == 0) return;
   Args a{};
-  a.n = n; a.K = m.K; a.KP = m.KP; a.rc = m.rc; a.accumulate = accumulate; a.arow = arow; a.acol = acol;
+  a.n = n; a.K = m.K; a.KP = m.KP; a.rc = m.rc; a.reach = m.L[t].reach; a.accumulate = accumulate; a.arow = arow; a.acol = acol;
   a.ar = ar; a.PHI = PHI; a.Wf = m.L[t].Wf; a.bf = m.L[t].bf; a.Gsm = Gsm; a.Gvm = Gvm; a.GPHI = GPHI;
   a.hedge = hedge; a.wst = const_cast<float*>(wst);
   CTD_DISPATCH(adj_go)
