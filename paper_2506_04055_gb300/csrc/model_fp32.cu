@@ -218,19 +218,33 @@ __global__ __launch_bounds__((BM / TM) * (BN / 4)) void k_gemm_small(
   }
 }
 
-// largest K of the tile shapes (3F = 768 at F = 256): 8 TM x 64 tiles up to TM = 4, above it, 16 x 32 tiles
+// largest K of the tile shapes (3F = 768 at F = 256): 8 TM x 64 tiles up to TM = 4 and 64 x 32 tiles, 8 TM x 64
+// above it, 16 x 32 tiles
 constexpr int kMidK = 512, kTallK = 384, kSmallK = 768;
 template <int EPI, int BM, int BN, int TM>
 static void launch_gemm_small(cudaStream_t st, int64_t M, int N, int K, const float* A, int lda, const float* B,
                               const float* bias, const float* aux, int ldaux, float* out, int ldo, float* out2, int ldo2) {
   static const cudaError_t attr = cudaFuncSetAttribute(
       k_gemm_small<EPI, BM, BN, TM>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-      (int)gemm_small_smem<BM, BN>(BN == 32 ? kSmallK : TM <= 4 ? kMidK : kTallK));
+      (int)gemm_small_smem<BM, BN>(BM == 16 ? kSmallK : TM <= 4 ? kMidK : kTallK));
   (void)attr;
   const unsigned grid = (unsigned)(((M + BM - 1) / BM) * ((N + BN - 1) / BN));
   LaunchScope ls_(st);
   k_gemm_small<EPI, BM, BN, TM><<<grid, (BM / TM) * (BN / 4), gemm_small_smem<BM, BN>(K), st>>>(
       M, N, K, A, lda, B, bias, aux, ldaux, out, ldo, out2, ldo2);
+}
+
+// The most 256-thread tiles of a problem for which the small tiles are faster: they pay one memory latency,
+// but a thread uses an operand for fewer outputs, so the line falls with K.  Measured on both sides of it
+// (us, small / 256-thread): N = 128, K = 64, 280 tiles 14.0 / 14.0; K = 128, 180 tiles 18.0 / 20.1, 200 tiles 22.1 / 20.1;
+// K = 256, 100 tiles 20.1 / 24.3, 120 tiles 28.3 / 24.3; K = 384, 80 tiles 32.4 / 34.4, 100 tiles 38.5 / 34.4; N = 256,
+// K = 768, 20 tiles 46.7 / 61.1, 40 tiles 75.4 / 61.1; narrow: N = 32, K = 64, 303 tiles 16.0 / 18.0, K = 256, 220 tiles
+// 42.7 / 52.9, 240 tiles 55.5 / 52.9.  (One line for every K, two waves, had cost N = 128, K = 384 at 19,000 rows
+// 100 against 51.)
+template <int BN>
+static int most_small_tiles(int K) {
+  if (BN == 32) return K <= 192 ? 304 : K <= 256 ? 220 : K <= 512 ? 180 : 25;
+  return K <= 64 ? 288 : K <= 192 ? 190 : K <= 256 ? 110 : K <= 384 ? 90 : K <= 512 ? 70 : 25;
 }
 
 template <int EPI, int BN>
@@ -239,8 +253,14 @@ static void gemm_tiled(cudaStream_t st, int64_t M, int N, int K, const float* A,
   if (M == 0) return;
   constexpr int BM = 8 * (256 / (BN / 4));
   const int64_t tiles = (int64_t)((N + BN - 1) / BN) * ((M + BM - 1) / BM);
-  if (tiles < 2 * 152 && K <= kSmallK) {   // under two waves of the 256-thread tiles
+  if (tiles <= most_small_tiles<BN>(K) && K <= kSmallK) {
     const int64_t cols = (N + 63) / 64, mid = ((M + 31) / 32) * cols;
+    // narrow outputs: 64 x 32 tiles (M = 45,000, N = 32, K = 64: 14 us; 64-wide tiles, half of their columns
+    // idle, 18; the 256 x 32 tiles 18)
+    if (BN == 32 && mid >= 152 && K <= kMidK) {
+      launch_gemm_small<EPI, 64, 32, 4>(st, M, N, K, A, lda, B, bias, aux, ldaux, out, ldo, out2, ldo2);
+      return;
+    }
     // 8 TM x 64 tiles once 32 rows of them fill the SMs, 16 x 32 tiles below that.  All tiles of an
     // SM run together, so a launch takes as long as the SM with the most: TM is the height whose
     // tiles per SM, times their work, is least (1.5 rows for what does not grow with TM): 5,997 atoms,
