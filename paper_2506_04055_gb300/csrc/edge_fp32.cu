@@ -100,9 +100,9 @@ constexpr int kBatch = 8;              // edges whose partials are reduced over 
 constexpr int kPartStride = 36;        // float4 per edge of a batch (32 lanes, padded: conflict-free)
 constexpr int64_t kChunkRows = 8;      // consecutive rows a warp group takes at a time, at most
 
-// Groups of four centres, and how many of the last ones keep their weights in registers.
+// How many of the last groups of four centres keep their weights in registers.
 template <int KR>
-constexpr int reg_groups() { return KR > 20 ? 4 : 3; }
+constexpr int reg_groups() { return KR > 20 ? 4 : KR >= 12 ? 3 : KR / 4; }
 
 struct Args {
   int64_t n, nchunks;
@@ -617,7 +617,7 @@ __global__ __launch_bounds__(32 * W, 1) void k_edge_adj(const __grid_constant__ 
 // Warps of a block (one block per SM): what the registers allow, 168 a thread for twelve warps and
 // 255 for eight.  Twelve of the wide kernels spill (adjoint, F = 64, 24,000 atoms: 698 us against 455).
 template <int KR, int F, int FPL, bool L0>
-constexpr int warps() { return L0 && KR <= 20 ? 12 : 8; }
+constexpr int warps() { return (L0 && KR <= 20) || KR <= 8 ? 12 : 8; }
 template <int KR, int F, int FPL, int W, bool STORE>
 constexpr size_t msg_smem() {
   return sizeof(float4) * 3 * Filter<KR, F, FPL>::NL * F +
@@ -686,8 +686,10 @@ void adj_go(cudaStream_t st, Args& a, bool first) {
     case 128: GO<KR, 128, 2>(st, a, t == 0); break; \
     default: GO<KR, 256, 2>(st, a, t == 0); break;  \
   }
+// Basis sizes are rounded up to 8, 16, 20 or 32 centres
 #define CTD_DISPATCH(GO)                     \
-  if (m.KP <= 16) { CTD_WIDTH(GO, 16) }      \
+  if (m.KP <= 8) { CTD_WIDTH(GO, 8) }        \
+  else if (m.KP <= 16) { CTD_WIDTH(GO, 16) } \
   else if (m.KP <= 20) { CTD_WIDTH(GO, 20) } \
   else { CTD_WIDTH(GO, 32) }
 
