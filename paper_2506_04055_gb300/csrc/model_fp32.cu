@@ -224,13 +224,13 @@ constexpr int kMidK = 512, kTallK = 384, kSmallK = 768;
 template <int EPI, int BM, int BN, int TM>
 static void launch_gemm_small(cudaStream_t st, int64_t M, int N, int K, const float* A, int lda, const float* B,
                               const float* bias, const float* aux, int ldaux, float* out, int ldo, float* out2, int ldo2) {
-  static const cudaError_t attr = cudaFuncSetAttribute(
-      k_gemm_small<EPI, BM, BN, TM>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-      (int)gemm_small_smem<BM, BN>(BM == 16 ? kSmallK : TM <= 4 ? kMidK : kTallK));
-  (void)attr;
   const unsigned grid = (unsigned)(((M + BM - 1) / BM) * ((N + BN - 1) / BN));
+  const size_t smem = gemm_small_smem<BM, BN>(K);
+  if (smem > 48 * 1024)   // the opt-in belongs to the current device; always the most, as threads share it
+    cudaFuncSetAttribute(k_gemm_small<EPI, BM, BN, TM>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                         (int)gemm_small_smem<BM, BN>(BM == 16 ? kSmallK : TM <= 4 ? kMidK : kTallK));
   LaunchScope ls_(st);
-  k_gemm_small<EPI, BM, BN, TM><<<grid, (BM / TM) * (BN / 4), gemm_small_smem<BM, BN>(K), st>>>(
+  k_gemm_small<EPI, BM, BN, TM><<<grid, (BM / TM) * (BN / 4), smem, st>>>(
       M, N, K, A, lda, B, bias, aux, ldaux, out, ldo, out2, ldo2);
 }
 
@@ -837,9 +837,7 @@ static size_t readout_fused_smem() {
 template <int F, int TA>
 static void launch_readout_fused(cudaStream_t st, const ModelW& m, int64_t n, const float* S_T, const float* ew, float* gs,
                                  float* e_atom, double* partials, int n_partials) {
-  static const cudaError_t attr = cudaFuncSetAttribute(
-      k_readout_fused<F, TA>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)readout_fused_smem<F, TA>());
-  (void)attr;
+  cudaFuncSetAttribute(k_readout_fused<F, TA>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)readout_fused_smem<F, TA>());
   LaunchScope ls_(st);
   k_readout_fused<F, TA><<<n_partials, 4 * TA, readout_fused_smem<F, TA>(), st>>>(n, m.e_scale, S_T, m.R1, m.R1t, m.d1, m.R2,
                                                                                  m.d2, ew, gs, e_atom, partials);
