@@ -208,8 +208,9 @@ int ctd_md_set_thermostat_state(ctd_ctx *ctx, const double *xi, const double *vx
  * filter (0). */
 #define CTD_OPT_TC_MESSAGE 3
 /* CTD_OPT_EDGE_CHUNK_ROWS (value >= 0; default 32): the tensor-core adjoint hands out the
- * sorted rows in chunks of this many rows, block-cyclically over all row streams of the GPU;
- * 0 gives each stream one contiguous range. */
+ * sorted rows in chunks of at most this many rows, cut evenly, block-cyclically over all row
+ * streams of the GPU; 0 gives each stream one contiguous range.  Values from 1 to 30 also bound the
+ * chunks of the tensor-core message step, which holds at most 16 rows otherwise. */
 #define CTD_OPT_EDGE_CHUNK_ROWS 4
 int ctd_set_option(ctd_ctx *ctx, int32_t option, int64_t value);
 
