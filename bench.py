@@ -48,11 +48,13 @@ def step_bytes_per_atom(n_e, value_bytes):
     return 42 * F * T * value_bytes + 2 * T * n_e * 8
 
 
-# FMA-pipe FLOPs per (active edge, feature channel) the edge kernels execute on CUDA cores
-# (reported beside the roofline): FP32 message 6K + 18, FP32 adjoint 12K + 45; with the filter
-# on the tensor pipe (BF16, F = 128, the cutoff and bias folded into the basis so the MMA yields
-# the filter and its derivative) the adjoint keeps 35 (the tensor-core message kernel's CUDA-core
-# work is per receiver, counted where it is reported).
+# FMA-pipe FLOPs per (active edge, feature channel) on CUDA cores (reported beside the roofline).
+# FP32 message 6K + 18, FP32 adjoint 12K + 45: the work of the full basis in a layer after the first.
+# The FP32 kernels execute less, since they leave out the Gaussians that are lost in the rounding
+# (about 6 of 20) and the first layer's zeros, so a rate from these is one of the full basis's work.
+# With the filter on the tensor pipe (BF16, F = 128, the cutoff and bias folded into the basis so
+# the MMA yields the filter and its derivative) the adjoint executes 35 (the tensor-core message
+# kernel's CUDA-core work is per receiver, counted where it is reported).
 EDGE_FWD_FLOP_PER_EF = 6 * K + 18
 EDGE_BWD_FLOP_PER_EF = 12 * K + 45
 EDGE_BWD_TC_ALU_FLOP_PER_EF = 35
@@ -430,7 +432,8 @@ def run_ours(args):
                                  else EDGE_FWD_FLOP_PER_EF)
         fma_peak = N_SM * FP32_LANES_PER_SM * 2 * peaks.get("sm_max_mhz", 2070.0) * 1e6 / 1e12
         roofline["fma_pipe"] = {"flop_per_launch": alu_flop, "tflops": alu_flop / launch_s / 1e12,
-                                "frac_of_fp32_fma_peak": alu_flop / launch_s / 1e12 / fma_peak}
+                                "frac_of_fp32_fma_peak": alu_flop / launch_s / 1e12 / fma_peak,
+                                "work": "executed" if tc else "full basis in every layer, of which part is not executed"}
     # the whole step against both roofs (algorithmic FLOPs and bytes per atom-step)
     step_s = s["ms_per_step"] / 1e3
     vb = 2 if head == "bf16" else 4
