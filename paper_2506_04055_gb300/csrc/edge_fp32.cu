@@ -34,9 +34,9 @@
 // (two FFMA without a reused operand 3.6), and each other instruction among them about two, which
 // makes the measured 208 (adjoint) and 106 (message) warp instructions per edge at F = 64 107 and 59
 // cycles of an SM; taking two edges at once or more warps changes nothing.
-// 96,000-atom water, F = 64, per launch: adjoint 1.80 ms (first layer 1.18), message 1.01 (0.67); one
-// thread per channel and all 20 centres took 2.76 and 1.41.  32,000-atom fcc, F = 128: 0.84 (0.50) and
-// 0.48 (0.30) against 1.26 and 0.68.
+// 96,000-atom water, F = 64, per launch: adjoint 1.82 ms (first layer 1.19), message 1.02 (0.67); one
+// thread per channel and all 20 centres took 2.76 and 1.41.  32,000-atom fcc, F = 128: 0.80 (0.49) and
+// 0.46 (0.29) against 1.26 and 0.68.
 // Every sum runs in an order that depends on the row alone (a row's edges in list order, an edge's
 // features in a fixed tree), so results do not depend on which rows share a launch.
 #include "ctd_internal.cuh"
