@@ -267,17 +267,23 @@ int prune_begin(ctd_ctx* c, double* maxdisp_out) {
   return CTD_OK;
 }
 
-// The buffers of a forces step whose size follows the Verlet list.  Grown by every step before its work
-// is recorded or replayed: a replay runs no checks, and a list may have been built (by a call that only
-// builds, or by one that failed after its build) since these were last sized.
-int ensure_edge_buffers(ctd_ctx* c) {
+static int ensure_active_list(ctd_ctx* c) {
   const int64_t e1 = c->n_verlet > 0 ? c->n_verlet : 1;
   ENSURE(c, c->acol, sizeof(int32_t) * e1);
   ENSURE(c, c->ar, sizeof(float4) * e1);
   ENSURE(c, c->vidx, sizeof(int32_t) * e1);
   ENSURE(c, c->arev, sizeof(int32_t) * e1);
   ENSURE(c, c->aend, sizeof(int32_t) * e1);
-  ENSURE(c, c->hedge, sizeof(float4) * e1);
+  return CTD_OK;
+}
+
+// The buffers of a forces step whose size follows the Verlet list, in the order in which an eager step
+// grows them.  For a step that is about to be recorded or replayed: a replay runs no checks, and a list may have been
+// built (by a call that only builds, or by one that failed after its build) since these were last sized.
+int ensure_edge_buffers(ctd_ctx* c) {
+  const int r = ensure_active_list(c);
+  if (r) return r;
+  ENSURE(c, c->hedge, sizeof(float4) * (c->n_verlet > 0 ? c->n_verlet : 1));
   return CTD_OK;
 }
 
@@ -288,7 +294,7 @@ int prune_finish(ctd_ctx* c) {
   const int64_t n = c->n, n1 = n > 0 ? n : 1;
   ENSURE(c, c->acount, sizeof(int32_t) * n1);
   ENSURE(c, c->arow, sizeof(int32_t) * (n1 + 1));
-  const int r = ensure_edge_buffers(c);
+  const int r = ensure_active_list(c);
   if (r) return r;
   const float rc2 = (float)(c->desc.rc * c->desc.rc);
   const uint8_t* near = c->use_near ? P<uint8_t>(c->near) : nullptr;
@@ -479,11 +485,14 @@ int forces_step(ctd_ctx* c, bool need_grad, bool gather_z) {
   if (c->local() || c->n == 0 || c->desc.T == 0 || c->n * c->desc.F > kGraphFeatures || prof_recording() ||
       model_stores_edges(c->mw, c->desc.precision))
     return body();
-  const int grown = ensure_edge_buffers(c);   // before the key: growth changes it
-  if (grown) return grown;
   using Act = decltype(c->records)::Act;
   const uint64_t key = key_now();
   Act act = c->records.next(key);
+  if (act != Act::kEager) {
+    const int r = ensure_edge_buffers(c);
+    if (r) return r;
+    if (key_now() != key) act = Act::kEager;   // one of them has grown
+  }
   if (act == Act::kRecord) {
     auto* rec = new RecordedStep();
     cudaGraph_t g = nullptr;

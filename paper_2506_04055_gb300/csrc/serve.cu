@@ -788,9 +788,12 @@ int ctd_serve_step(ctd_server* s, int32_t* n_resident, int32_t* n_admitted, int3
   CUDA_OK(c, cudaMemsetAsync(c->status.p, 0, sizeof(int32_t), st));
   const bool graphable = s->use_graph && !c->local() && !prof_recording() &&
                          !model_stores_edges(c->mw, c->desc.precision);
-  // a replay runs no buffer checks: what is sized by the lists grows here, which changes the key
-  if (int r = ensure_edge_buffers(c)) return r;
-  const uint64_t key = layout_key(s, nres);
+  uint64_t key = layout_key(s, nres);
+  if (graphable && ((s->gexec && s->gkey == key) || key == s->last_key)) {
+    // a replay runs no buffer checks: what is sized by the lists grows here, which changes the key
+    if (int r = ensure_edge_buffers(c)) return r;
+    key = layout_key(s, nres);
+  }
   bool launched = false;
   if (graphable && s->gexec && s->gkey == key) {
     CUDA_OK(c, cudaGraphLaunch(s->gexec, st));

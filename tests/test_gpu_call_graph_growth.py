@@ -60,7 +60,8 @@ def test_denser_system_under_a_recorded_step(F, prec, how):
 
 
 def test_growth_under_a_budget():
-    """Budgets from too small to ample: every call gives the eager result or reports the budget."""
+    """Budgets from too small to ample: every call gives the eager result or reports the budget, and a context
+    whose steps are recorded takes exactly the budgets that an eager one takes."""
     eng = engine()
     from paper_2506_04055_gb300 import _lib
     dense = syn.fcc(5, 5, 10, jitter=0.05, seed=3)
@@ -72,16 +73,25 @@ def test_growth_under_a_budget():
         _build_large(pot, "build")
         held = [pot.compute(dense.species, p, c, stats=True)["stats"]["bytes_allocated"]
                 for p, c in ((x, cell), (dense.positions, dense.cell))]
-    refused = 0
-    for budget in np.linspace(0.5 * held[0], 1.03 * held[1], 25).astype(int):
+
+    def calls_done(budget, eager):
+        done = 0
         with eng.Potential(64, T=2, n_species=1, params=blob, hbm_budget_bytes=int(budget)) as pot:
+            pot.profile(eager)
             try:
                 _build_large(pot, "build")
                 for _ in range(5):
                     _same(pot.compute(dense.species, x, cell, energies=True), thin)
+                    done += 1
                 for _ in range(3):
                     _same(pot.compute(dense.species, dense.positions, dense.cell, energies=True), want)
+                    done += 1
             except _lib.CtdError as e:
                 assert e.code == _lib.CTD_ERR_OUT_OF_BUDGET
-                refused += 1
-    assert 0 < refused < 25
+        return done
+
+    counts = []
+    for budget in np.linspace(0.5 * held[0], 1.03 * held[1], 60).astype(int):
+        counts.append(calls_done(budget, False))
+        assert counts[-1] == calls_done(budget, True), budget
+    assert counts[0] == 0 and counts[-1] == 8
