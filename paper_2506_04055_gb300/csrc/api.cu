@@ -703,6 +703,7 @@ int load_params_impl(ctd_ctx* c, const void* blob, size_t nbytes) {
   const int KP = (K + 3) / 4 * 4;
   // host staging of every FP32 array, 16-byte aligned offsets
   std::vector<float> h;
+  h.reserve((size_t)nval * 2 + (size_t)T * 3 * F * 72 + 4096);   // most matrices twice, and the padded filters
   auto alloc = [&](size_t cnt) {
     size_t off = (h.size() + 7) / 8 * 8;   // 32 B: the BF16 twin of every array is 16-byte aligned
     h.resize(off + cnt, 0.0f);
@@ -791,11 +792,12 @@ int load_params_impl(ctd_ctx* c, const void* blob, size_t nbytes) {
   const __nv_bfloat16* bbase = P<__nv_bfloat16>(c->params_bf);
   // FP16 copies of the zero-padded radial filters [3F][64] for the tensor-core adjoint; a filter
   // weight beyond FP16's range keeps that model on the CUDA-core adjoint (FP32 weights)
-  std::vector<__half> hh((size_t)T * 3 * F * 64);
+  std::vector<__half> hh((size_t)T * 3 * F * 64, __float2half_rn(0.0f));
   bool f16_ok = true;
   for (int t = 0; t < T; ++t)
     for (size_t k = 0; k < (size_t)3 * F * 64; ++k) {
       const float x = h[lo[t].Wf64 + k];
+      if (x == 0.0f) continue;   // most of it is padding
       if (!(std::fabs(x) <= 65504.0f)) f16_ok = false;
       hh[(size_t)t * 3 * F * 64 + k] = __float2half_rn(x);
     }
